@@ -47,7 +47,7 @@ typedef enum {
     HP_ERR_NONFINITE = 3,   /* the input velocity holds NaN or Inf */
     HP_ERR_OOM = 5,         /* device allocation failed */
     HP_ERR_UNSUPPORTED = 6, /* the requested combination is not built */
-    HP_ERR_TIMEOUT = 7,     /* a tensor-core completion wait gave up (hp_cnn_check) */
+    HP_ERR_TIMEOUT = 7,     /* a bounded device wait gave up (hp_cnn_check, hp_ctx_check) */
     HP_ERR_IO = 8,          /* a checkpoint file could not be written, or is missing,
                                truncated, corrupted or of another format version */
     HP_ERR_GUARD = 9,       /* a workspace's guard zone was overwritten (hp_ctx_check,
@@ -84,11 +84,10 @@ typedef struct {
  *                  2 = temporally blocked (T
  *                  sweeps per launch, replay to the exact stop; 4 rows per
  *                  thread), 3 = temporally blocked with 2 rows per thread
- *                  (twice the warps), 4 = grid-resident: one thread-block
- *                  cluster (up to 16 CTAs of 128 x 128 cells) keeps a whole
- *                  grid on chip for all sweeps, falling back to 2 when the
- *                  grid is larger than 512 x 512 cells or the cluster does
- *                  not fit on the device.  All give the same iterates bit for
+ *                  (twice the warps), 4 = grid-resident: strips of whole
+ *                  rows on up to all SMs of the device keep a grid on chip
+ *                  for all sweeps (grids up to 512 cells wide), falling back
+ *                  to 2 for wider grids.  All give the same iterates bit for
  *                  bit; the FP64 E_k may differ in the last bits between
  *                  kernels (their partial sums are grouped differently).
  *   open_top       1 = the top boundary (the v faces of row 0) is open to an
@@ -130,7 +129,8 @@ void hp_ctx_destroy(hp_ctx *ctx);
  * bytes longer and those guard bytes hold a fixed pattern; this call
  * synchronises the device and returns HP_ERR_GUARD if a kernel wrote into a
  * guard zone (past the end of a workspace), HP_ERR_CUDA on a pending CUDA
- * error, else HP_OK. */
+ * error, HP_ERR_TIMEOUT if a bounded wait of the sweep kernel gave up since
+ * the last check (its results are then void), else HP_OK. */
 hp_status hp_ctx_check(hp_ctx *ctx);
 
 const char *hp_status_string(hp_status s);
@@ -197,11 +197,11 @@ hp_status hp_jacobi_target(hp_ctx *ctx, const float *div, const uint8_t *flags, 
                            float *target_out, hp_shape shape, void *stream);
 
 /* Number of grids of this shape that the grid-resident sweep kernel
- * (sweep_kernel = 4) can hold on the device at once, one thread-block cluster
- * of ceil(nx/128) x ceil(ny/128) CTAs per grid; 0 when that kernel cannot run
- * the shape (grid above 512 x 512 cells, or the cluster does not fit), in
- * which case hp_project falls back to the temporally blocked kernel.  Host
- * query only (no kernel launch); 0 for a NULL context or an invalid shape. */
+ * (sweep_kernel = 4) holds on the device at once, each cut into strips of
+ * whole rows on one SM each (their height by the batch: the fewer grids, the
+ * more SMs per grid); 0 for grids above 512 x 512 cells (128 x 128 tiles
+ * beyond 16).  Host query only (no kernel launch); 0 for a NULL context or an
+ * invalid shape. */
 int32_t hp_resident_clusters(hp_ctx *ctx, hp_shape shape);
 
 /* Parameters of the plume driver step (Sec. 2.2: semi-Lagrangian advection

@@ -139,6 +139,8 @@ void hp_ctx_destroy(hp_ctx* c)
     cudaFree(c->partial2);
     cudaFree(c->gs);
     cudaFree(c->ls);
+    cudaFree(c->box);
+    cudaFree(c->wait_err);
     if (c->host_flag) cudaFreeHost(c->host_flag);
     if (prev >= 0) cudaSetDevice(prev);
     delete c;
@@ -183,7 +185,9 @@ hp_status hp_ctx_create(hp_ctx** out, hp_shape mx, int device)
         (rc = dalloc(&c->partial, c->partial_len, &c->guards)) != HP_OK ||
         (rc = dalloc(&c->partial2, c->partial2_len, &c->guards)) != HP_OK ||
         (rc = dalloc(&c->gs, (size_t)mx.batch, &c->guards)) != HP_OK ||
-        (rc = dalloc(&c->ls, 1, &c->guards)) != HP_OK) {
+        (rc = dalloc(&c->ls, 1, &c->guards)) != HP_OK ||
+        (rc = dalloc((uint8_t**)&c->box, resident_box_bytes(), &c->guards)) != HP_OK ||
+        (rc = dalloc(&c->wait_err, 1, &c->guards)) != HP_OK) {
         hp_ctx_destroy(c);
         return rc;
     }
@@ -214,7 +218,13 @@ hp_status hp_ctx_check(hp_ctx* c)
     if (!c) return HP_ERR_INVALID_ARG;
     cudaError_t e = cudaSetDevice(c->device);
     if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
-    return check_guards(c->guards);
+    hp_status rc = check_guards(c->guards);
+    if (rc != HP_OK) return rc;
+    int32_t gave_up = 0;
+    e = cudaMemcpy(&gave_up, c->wait_err, sizeof(gave_up), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && gave_up) e = cudaMemset(c->wait_err, 0, sizeof(gave_up));
+    if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
+    return gave_up ? HP_ERR_TIMEOUT : HP_OK;
 }
 
 hp_status hp_face_mask(const uint8_t* flags, uint8_t* mask_out, hp_shape s, void* stream)

@@ -43,7 +43,7 @@ struct GridState {
     int32_t src;         // buffer holding phi_{k0_stop}
     int32_t final_buf;   // buffer holding phi_{k*}
     int32_t converged;   // 1 when E(phi_{k*}) <= threshold
-    int32_t pad_;
+    uint32_t wild;       // epoch of the launch that found values beyond 1e20 in this grid
     double e_stop;       // E(phi_{k*})
     uint32_t arrivals;   // CTA arrival counter of the current launch
     uint32_t pad2_;
@@ -120,7 +120,9 @@ struct hp_ctx {
     hp::GridState* gs;
     hp::LoopState* ls;
     float* ckpt;         // [max_cells] checkpoint buffer of the resident sweep kernel
-    int res_clusters[17];  // per cluster size: 0 unknown, else 1 + clusters that fit
+    void* box;           // exchange area of the resident sweep kernel (ResBox)
+    int32_t* wait_err;   // set by a bounded wait of that kernel that gave up
+    uint32_t epoch;      // its launches
     int32_t* host_flag;  // pinned
     // cached conditional-graph loop
     cudaGraphExec_t graph_exec;
@@ -214,10 +216,11 @@ __device__ __forceinline__ uint32_t load_mask4(const uint8_t* __restrict__ row, 
 }
 
 void set_cuda_error(cudaError_t e);
-int resident_tiles(hp_shape s);
+size_t resident_box_bytes();
 int resident_capacity(hp_ctx* ctx, hp_shape s);
-hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int max_iters,
-                          double* e_hist, int hist_len, cudaStream_t st, bool* launched);
+hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bool fixed,
+                          const float* phi0, double* e_hist, int hist_len, cudaStream_t st,
+                          bool* launched);
 hp_status check_launch();
 bool shape_ok(hp_shape s);
 

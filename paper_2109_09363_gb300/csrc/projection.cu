@@ -325,9 +325,9 @@ __global__ void reset_state_kernel(GridState* gs, LoopState* ls, int B)
     }
 }
 
-// phi_0 = given guess on cells with an open face, else 0.
-__global__ void init_phi_kernel(const float* __restrict__ phi0, const uint8_t* __restrict__ mask,
-                                float* __restrict__ out, size_t cells)
+// phi_0 = given guess on cells with an open face, else 0 (out may be phi0).
+__global__ void init_phi_kernel(const float* phi0, const uint8_t* __restrict__ mask, float* out,
+                                size_t cells)
 {
     const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= cells) return;
@@ -1463,10 +1463,6 @@ hp_status project_impl(hp_ctx* ctx, float* u, float* v, const uint8_t* flags, hp
         rc = launch_mask_div(u, v, flags, ctx->mask, ctx->div, s, st, boundary_of(*prm));
         if (rc != HP_OK) return rc;
     }
-    init_phi_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(phi0, ctx->mask, ctx->phi[0],
-                                                                     cells);
-    if ((rc = check_launch()) != HP_OK) return rc;
-
     const bool fixed = prm->fixed_iters > 0;
     const int cap = fixed ? prm->fixed_iters : prm->max_iters;
     const double thr = fixed ? -1.0 : prm->threshold;
@@ -1479,12 +1475,13 @@ hp_status project_impl(hp_ctx* ctx, float* u, float* v, const uint8_t* flags, hp
         // library choice: the whole grid on chip, one cluster per grid
         // (measured 1.85x faster than the blocked kernel at 16 x 512^2); the
         // blocked loop when the grid is larger or the cluster does not fit
-        reset_state_kernel<<<(s.batch + 255) / 256, 256, 0, st>>>(ctx->gs, ctx->ls, s.batch);
-        if ((rc = check_launch()) != HP_OK) return rc;
-        rc = launch_resident(ctx, s, thr, cap, e_hist, hist_len, st, &resident);
+        rc = launch_resident(ctx, s, thr, cap, fixed, phi0, e_hist, hist_len, st, &resident);
         if (rc != HP_OK) return rc;
     }
     if (!resident) {
+        init_phi_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(phi0, ctx->mask,
+                                                                         ctx->phi[0], cells);
+        if ((rc = check_launch()) != HP_OK) return rc;
         rc = run_sweep_loop(ctx, s, pick_T(prm), R, stream, thr, cap, e_hist, hist_len,
                             prm->use_graph != 0, st);
         if (rc != HP_OK) return rc;

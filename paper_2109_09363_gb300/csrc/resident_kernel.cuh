@@ -1,0 +1,924 @@
+// Grid-resident masked Jacobi sweeps for sm_103a (Sec. 2.2 Jacobi iteration,
+// stop rule of Sec. 3.3 / 4.1): the kernel, instantiated by resident_*.cu.
+//
+// A grid stays on chip for all of its sweeps.  It is cut into horizontal
+// strips of whole rows, one CTA (one SM) each, up to 512 cells wide; the CTAs
+// of one grid form a group, and one cooperative launch holds as many groups as
+// fit on the device, each working through grids of the batch.  A CTA is 16
+// warps in WX columns of 32 C cells and 16 / WX warp rows; thread (warp, lane)
+// holds R rows x C columns of phi in registers, div and four bits of open-face
+// count per cell sit in shared memory.  Per sweep and warp:
+//   - the rows next to the warp's block come from shared memory (double
+//     buffered), or, at the edge of the strip, from the neighbouring CTA
+//     through the L2: every 32-bit value travels with the number of its
+//     message in one 64-bit word, so the receiver polls the data itself and
+//     no fence or flag is needed;
+//   - warps of the lower half hold their rows bottom up, so that the row at
+//     the strip's edge is register row 0 in every edge warp: it is computed
+//     and sent first, and travels while the other rows are computed; the
+//     receiver issues its load halfway through the sweep;
+//   - groups of rows whose cells all have the open-face count of an
+//     unobstructed row of that column take the update without the closed-face
+//     terms (bit for bit the same result: the left-out product is an exact
+//     zero), the others look 4 - n and 1/n up by the cell's bits.
+// The only barrier of a sweep is the CTA's own.
+//
+// E_k: FP32 |r| per thread and warp, then sums of float pairs (TwoSum, 48
+// bits; an FP64 addition of a warp occupies its scheduler's FP64 unit for 64
+// cycles here, and four dependent ones per round cost 0.6 us a sweep) per CTA
+// (16 warp sums) and per group (CTA partials in rank order), in rounds of four
+// sweeps.  Round q holds sweeps 4q..4q+3; one warp of every CTA posts the CTA
+// partials, rank 0 adds them one round later and posts the stop decision,
+// every CTA reads it one round after that, so all CTAs of a group leave the
+// loop at the same sweep and go back to the last checkpoint of phi at or below
+// k* (one every 32 sweeps), from which they replay the sweeps to k* exactly.
+// The comparison with the threshold is made in FP64 whenever the FP32 head of
+// the sum is within 1e-6 of it.  phi at the cap is kept aside as it passes, so
+// a grid that reaches its cap replays nothing; a run of fixed length needs
+// neither E nor a decision.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include "hproj_internal.cuh"
+
+namespace hp {
+
+constexpr int kResWarps = 8;       // sweep warps: two warpgroups
+constexpr int kResSweepers = kResWarps * 32;
+constexpr int kResThreads = kResSweepers + 128;  // and one of helpers
+constexpr int kResMaxCtas = 192;   // CTAs of one launch (one per SM)
+// registers a thread: 384 x 168 at launch, then 232 for the sweep warps and 40
+// for the helpers: 128 x (2 x 232 + 40) = 384 x 168
+constexpr int kResRegs = 168, kResRegsSweep = 232, kResRegsHelp = 40;
+static_assert(kResSweepers * kResRegsSweep + 128 * kResRegsHelp <= kResThreads * kResRegs,
+              "the split waits forever for registers the launch does not have");
+// a decision about sweep j is known everywhere before sweep 4 (j / 4 + kResLag)
+constexpr int kResLag = 3;
+constexpr int kResRing = 4;        // > kResLag: rounds between the sweeps and the decision
+constexpr int kWsumRing = 4 * kResRing;  // warp sums, by sweep
+// polls of a bounded wait before it gives up (each at least one L2 round
+// trip, so half a second or more); of a shared-memory wait
+constexpr int kResPolls = 1 << 20, kResSpins = 1 << 22;
+// the sums of pairs are scaled (exactly) so that no sum of finite warp sums overflows
+constexpr float kSumScale = 1.0f / 4096.0f;
+static_assert(kResMaxCtas * kResWarps <= 4096, "warp sums of one grid");
+
+// Exchange area in global memory (one per context, cleared before every
+// launch): messages between neighbouring CTAs, E partials, decisions, queue.
+struct ResBox {
+    // row messages: [receiver][side: from above, from below][parity]
+    uint4 row[kResMaxCtas][2][2][256];  // [word][lanes of the strip's width]
+    uint4 part[kResMaxCtas][kResRing][4];  // E partial of one sweep: head, tag, tail, tag
+    uint4 dec[kResMaxCtas][kResRing];      // by group: decision, tag, sweep, tag
+    uint4 next[kResMaxCtas][2];            // by group: grid, tag
+    uint32_t queue;                        // grids handed out beyond the first of each group
+};
+
+struct ResArgs {
+    const float* phi0;  // phi_0 of the caller (cells without an open face ignored), null = 0
+    float* phi;         // phi_{k*} out (may be phi0)
+    float* ck[2];       // checkpoint buffers [B][ny][nx]
+    const float* div;   // [B][ny][nx]
+    const uint8_t* mask;
+    GridState* gs;
+    ResBox* box;
+    int32_t* err;       // set to 1 when a wait gave up
+    double* e_hist;     // [B][hist_len] or null
+    int32_t hist_len;
+    int32_t B, ny, nx;
+    int32_t n;          // CTAs per grid
+    int32_t groups;
+    int32_t cap;
+    int32_t phi0_vec;   // phi0 allows 16-byte loads
+    uint32_t epoch;     // of this launch (GridState::wild)
+    int32_t fixed;      // exactly cap sweeps; E only for grids whose values could overflow
+    double threshold;   // < 0: never stops before the cap
+    float sum_near;     // sums of |r| above it are above the threshold
+};
+
+template <int C, int R, int WX>
+struct ResLayout {
+    static constexpr int WY = kResWarps / WX;
+    static constexpr int V = C / 4;                                      // 16-byte words per row
+    static constexpr int kDiv = 0;                                       // [16][R][V][32] float4
+    static constexpr int kCode = kDiv + kResWarps * R * V * 512;         // [16][R][32] u32, 4 bits a cell
+    // rows next to a block: [2 parities][16 warps x 2 rows + a zero row][V][32] float4
+    static constexpr int kRow = kCode + kResWarps * R * 128;
+    static constexpr int kRowSlot = V * 512;
+    static constexpr int kRowPar = (2 * kResWarps + 1) * kRowSlot;
+    // columns next to a block: [2][16 warps x 2 columns + a zero column][R] float
+    static constexpr int kCol = kRow + 2 * kRowPar;
+    static constexpr int kColPar = (2 * kResWarps + 1) * R * 4;
+    // rows received from the neighbouring CTAs: [2 sides][2 parities][WX][V][32] float4
+    static constexpr int kHalo = kCol + 2 * kColPar;
+    static constexpr int kHaloPar = WX * kRowSlot;
+    static constexpr int kLut = kHalo + 4 * kHaloPar;                    // [5] float2
+    static constexpr int kWsum = kLut + 64;                              // [16][8] float
+    static constexpr int kBytes = kWsum + kWsumRing * kResWarps * 4;
+    static_assert(R % 4 == 0 && C % 4 == 0, "rows and columns go out four values at a time");
+    static_assert(kBytes <= 227 * 1024 - 64, "shared memory of one CTA");
+};
+
+// ---- 16-byte words through the L2 (each 8-byte half holds a value and its tag)
+
+__device__ __forceinline__ uint4 ld_box(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_box(uint4* p, uint32_t a, uint32_t b, uint32_t tag)
+{
+    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a), "r"(tag),
+                 "r"(b), "r"(tag)
+                 : "memory");
+}
+
+// ---- barriers in shared memory
+__device__ __forceinline__ uint32_t res_smem(const void* p)
+{
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+__device__ __forceinline__ void bar_init(uint64_t* b, int count)
+{
+    asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(res_smem(b)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void bar_arrive(uint64_t* b)
+{
+    asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.shared.b64 t, [%0];\n\t}" ::"r"(res_smem(b))
+                 : "memory");
+}
+
+// whether the phase of this parity has completed; bounded
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, int spins)
+{
+    uint32_t done = 0;
+    do {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(res_smem(b)), "r"(parity)
+            : "memory");
+    } while (!done && --spins > 0);
+    return done != 0;
+}
+
+// named barriers: 1 the sweep warps, 2 these and the helper of the E rounds
+__device__ __forceinline__ void sync_sweepers()
+{
+    asm volatile("barrier.cta.sync 1, %0;" ::"n"(kResSweepers) : "memory");
+}
+__device__ __forceinline__ void sync_grid()
+{
+    asm volatile("barrier.cta.sync 2, %0;" ::"n"(kResSweepers + 32) : "memory");
+}
+
+// ---- sums of float pairs: h + l, |l| <= ulp(h) / 2 (TwoSum, Knuth)
+struct Pair {
+    float h, l;
+};
+
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b)
+{
+    const float s = __fadd_rn(a.h, b.h);
+    const float t = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+    const float f = __fadd_rn(e, __fadd_rn(a.l, b.l));
+    const float h = __fadd_rn(s, f);
+    return {h, __fsub_rn(f, __fsub_rn(h, s))};
+}
+
+// over the eight lanes of a group, result in its first lane
+__device__ __forceinline__ Pair pair_tree(Pair v)
+{
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+        const Pair o = {__shfl_down_sync(0xffffffffu, v.h, off, 8),
+                        __shfl_down_sync(0xffffffffu, v.l, off, 8)};
+        v = pair_add(v, o);
+    }
+    return v;
+}
+
+template <int C, int R, int WX>
+struct ResWarp {
+    using L = ResLayout<C, R, WX>;
+    static constexpr int V = C / 4;
+    uint8_t* sm;
+    int lane, wid, wx, wy;
+    bool flip;        // register row r is image row y0 + R - 1 - r
+    bool rem;         // the row beside register row 0 comes from another CTA
+    bool out;         // this lane lies right of the grid
+    uint32_t gen;     // bit g: some cell of rows 4g..4g+3 differs from its column's default
+    uint32_t skip;    // bit g: rows 4g..4g+3 lie outside the grid
+    float c0, inv0, invm, inv3, c3;  // column defaults (first, inner and last cell; inner c = 0)
+    int in_f, in_l;   // byte offsets (parity 0) of the rows beside rows 0 and R - 1
+    int in_c;         // of the column beside this lane's edge (left, lane 31: right)
+    int out_r, out_c; // of this warp's own rows and column
+    int in_h;         // of the row received from the neighbouring CTA
+    uint64_t* full;   // [parity]: it is there
+    uint4* tx;        // [parity][word] to the neighbouring CTA, this lane
+    uint32_t t;       // messages sent (= received and being waited for) so far
+    bool dead;        // a wait gave up: do not wait any more
+
+    __device__ __forceinline__ void ld_row(int off, float (&v)[C]) const
+    {
+#pragma unroll
+        for (int h = 0; h < V; ++h) {
+            const float4 f = *reinterpret_cast<const float4*>(sm + off + 512 * h);
+            v[4 * h] = f.x; v[4 * h + 1] = f.y; v[4 * h + 2] = f.z; v[4 * h + 3] = f.w;
+        }
+    }
+    __device__ __forceinline__ void st_row(int off, const float (&v)[C]) const
+    {
+#pragma unroll
+        for (int h = 0; h < V; ++h)
+            *reinterpret_cast<float4*>(sm + off + 512 * h) =
+                make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+    }
+    static constexpr int kMsgLanes = 32 * WX;
+    // the row of message t, from the helper that receives it; bounded
+    __device__ __forceinline__ void receive(float (&v)[C], int32_t* err)
+    {
+        if (!bar_wait(full + (t & 1u), (t - 1) >> 1 & 1u, dead ? 1 : kResSpins)) {
+            dead = true;
+            *err = 1;
+        }
+        ld_row(in_h + (t & 1u ? L::kHaloPar : 0), v);
+    }
+    __device__ __forceinline__ void send(const float (&v)[C], uint32_t tag) const
+    {
+        uint4* p = tx + (tag & 1u) * 256;
+#pragma unroll
+        for (int i = 0; i < 2 * V; ++i)
+            st_box(p + kMsgLanes * i, __float_as_uint(v[2 * i]), __float_as_uint(v[2 * i + 1]), tag);
+    }
+    // boundary values of phi into the buffers of message t + 1
+    __device__ __forceinline__ void publish(const float (&phi)[R][C])
+    {
+        ++t;
+        const int pr = (t & 1u) ? L::kRowPar : 0, pc = (t & 1u) ? L::kColPar : 0;
+        st_row(out_r + pr, phi[0]);
+        st_row(out_r + pr + L::kRowSlot, phi[R - 1]);
+        if (rem) send(phi[0], t);
+        if (WX > 1) {
+#pragma unroll
+            for (int r = 0; r < R; r += 4) {
+                const bool q = lane == 31;
+                const float4 c = make_float4(
+                    q ? phi[r][C - 1] : phi[r][0], q ? phi[r + 1][C - 1] : phi[r + 1][0],
+                    q ? phi[r + 2][C - 1] : phi[r + 2][0], q ? phi[r + 3][C - 1] : phi[r + 3][0]);
+                if (lane == 0 || lane == 31)
+                    *reinterpret_cast<float4*>(sm + out_c + pc + 4 * r) = c;
+            }
+        }
+    }
+    // every message is received, also the one no sweep uses: the sender counts on it
+    __device__ __forceinline__ void drain(int32_t* err)
+    {
+        if (rem) {
+            float v[C];
+            receive(v, err);
+        }
+    }
+
+    // phi_{k+1} from phi_k and the boundary values of message t; sends message
+    // t + 1.  WITH_E: `pending` (this thread's FP32 sum of |r(phi_{k-1})|) is
+    // summed over the warp while the rows are computed, stored in *wsum by lane
+    // 0, and becomes the sum of |r(phi_k)|.
+    template <bool WITH_E>
+    __device__ __forceinline__ void update(float (&phi)[R][C], float& pending, float* wsum,
+                                           int32_t* err)
+    {
+        const int pr = (t & 1u) ? L::kRowPar : 0, pc = (t & 1u) ? L::kColPar : 0;
+        const int qr = L::kRowPar - pr, qc = L::kColPar - pc;
+        // a warp-wide OR lands in a uniform register: the branches below stay
+        // uniform (a fifth of the instructions were their divergence handling)
+        const uint32_t cls = __reduce_or_sync(0xffffffffu, gen | skip << 8 | (rem ? 1u << 16 : 0u));
+        const uint32_t any = cls | cls >> 8;
+        const bool far = (cls >> 16) != 0;
+        // ds of the row before: south difference, the negated north one of this row
+        float dsp[C];
+        if (far) receive(dsp, err);
+        else ld_row(in_f + pr, dsp);
+#pragma unroll
+        for (int q = 0; q < C; ++q) dsp[q] = __fsub_rn(phi[0][q], dsp[q]);
+        const int s_div = L::kDiv + (wid * R * V * 32 + lane) * 16;
+        const int s_code = L::kCode + (wid * R * 32 + lane) * 4;
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float s = pending;
+        // one row: differences of phi_k (each formed once: south of row r is
+        // minus north of row r + 1, east of a cell minus west of the next),
+        // then the update in one of two forms
+        auto row = [&](auto plain, int r, float halo) {
+            float d[C];
+            ld_row(s_div + r * L::kRowSlot, d);
+            float left = __shfl_up_sync(0xffffffffu, phi[r][C - 1], 1);
+            float right = __shfl_down_sync(0xffffffffu, phi[r][0], 1);
+            if (lane == 0) left = halo;
+            if (lane == 31) right = halo;
+            float below[C];
+            if (r + 1 == R) ld_row(in_l + pr, below);
+            float exw = __fsub_rn(phi[r][0], left);
+            uint32_t even = 0, odd = 0;  // 8 n of the even and of the odd cells, a byte each
+            if (!plain.value) {
+                const uint32_t code = *reinterpret_cast<const uint32_t*>(sm + s_code + r * 128);
+                even = (code << 3) & 0x78787878u;
+                odd = (code >> 1) & 0x78787878u;
+            }
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                const float pc0 = phi[r][q];
+                const float exe = __fsub_rn(q + 1 < C ? phi[r][q + 1] : right, pc0);
+                const float ds = __fsub_rn(r + 1 < R ? phi[r + 1 < R ? r + 1 : r][q] : below[q], pc0);
+                float lap = __fadd_rn(__fsub_rn(exe, exw), __fsub_rn(ds, dsp[q]));
+                exw = exe;
+                dsp[q] = ds;
+                float res;
+                if (plain.value) {
+                    float inv = invm;
+                    if (q == 0) {
+                        lap = __fmaf_rn(c0, pc0, lap);
+                        inv = inv0;
+                    } else if (q == C - 1) {
+                        lap = __fmaf_rn(c3, pc0, lap);
+                        inv = inv3;
+                    }
+                    res = __fsub_rn(d[q], lap);
+                    phi[r][q] = __fmaf_rn(-res, inv, pc0);
+                } else {
+                    const float2 k = *reinterpret_cast<const float2*>(
+                        sm + L::kLut + (((q & 1 ? odd : even) >> (8 * (q / 2))) & 0xffu));
+                    // [n > 0] from 1/n in {0, 1/4, 1/3, 1/2, 1}: saturate(4/n) is 0 or 1
+                    lap = __fmaf_rn(k.x, pc0, lap);
+                    res = __fmaf_rn(-__saturatef(k.y * 4.0f), lap, d[q]);
+                    phi[r][q] = __fmaf_rn(-res, k.y, pc0);
+                }
+                if (WITH_E) acc[q % 4] = __fadd_rn(acc[q % 4], fabsf(res));
+            }
+        };
+#pragma unroll
+        for (int g = 0; g < R / 4; ++g) {
+            float h[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if (WX > 1) {
+                const float4 hv = *reinterpret_cast<const float4*>(sm + in_c + pc + 16 * g);
+                h[0] = hv.x; h[1] = hv.y; h[2] = hv.z; h[3] = hv.w;
+            }
+            // after row i of the group: the boundary rows go out, a level of
+            // the warp sum of the sweep before
+            auto after = [&](int i) {
+                const int r = 4 * g + i;
+                if (r == 0) {
+                    if (far) send(phi[0], t + 1);
+                    st_row(out_r + qr, phi[0]);
+                }
+                if (r == R - 1) st_row(out_r + qr + L::kRowSlot, phi[R - 1]);
+            };
+            if (WITH_E) {
+#pragma unroll
+                for (int i = 0; i < 5; ++i) {  // five levels over the groups there are
+                    if (i * (R / 4) / 5 == g)
+                        s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 16 >> i));
+                }
+            }
+            if (!(any & (1u << g))) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    row(Bool<true>{}, 4 * g + i, h[i]);
+                    after(i);
+                }
+            } else if (!(cls & (256u << g))) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    row(Bool<false>{}, 4 * g + i, h[i]);
+                    after(i);
+                }
+            } else {  // phi stays 0; the next group's north differences
+#pragma unroll
+                for (int q = 0; q < C; ++q)
+                    dsp[q] = 4 * g + 4 < R ? phi[4 * g + 4 < R ? 4 * g + 4 : 0][q] : 0.0f;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) after(i);
+            }
+            if (WX > 1) {
+                const bool q = lane == 31;
+                // predicated, not branched around
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\t"
+                    "@p st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n\t}" ::"r"(
+                        (uint32_t)__cvta_generic_to_shared(sm + out_c + qc + 16 * g)),
+                    "f"(q ? phi[4 * g][C - 1] : phi[4 * g][0]),
+                    "f"(q ? phi[4 * g + 1][C - 1] : phi[4 * g + 1][0]),
+                    "f"(q ? phi[4 * g + 2][C - 1] : phi[4 * g + 2][0]),
+                    "f"(q ? phi[4 * g + 3][C - 1] : phi[4 * g + 3][0]),
+                    "r"((int)(lane == 0 || q))
+                    : "memory");
+            }
+        }
+        ++t;
+        if (WITH_E) {
+            if (lane == 0) *wsum = s;
+            pending = out ? 0.0f
+                          : __fadd_rn(__fadd_rn(acc[0], acc[1]), __fadd_rn(acc[2], acc[3]));
+        }
+    }
+    template <bool P>
+    struct Bool {
+        static constexpr bool value = P;
+    };
+};
+
+// Shared by the sweep warps and the helpers of one CTA.
+struct ResShared {
+    uint64_t full[2][2];       // [side][parity]: a neighbour's row is there
+    uint64_t sums[kResRing];   // the warp sums of a round are there
+    volatile uint32_t end;     // messages in all, once the CTA is done
+    volatile int rounds;       // rounds of this grid decided
+    volatile int stop;         // the round that stopped it
+    int kstar, code;           // k*; 1 converged, 2 not
+    double estar;
+    int act;                   // 1: leave the sweep loop
+    int grid;                  // next grid of the group
+};
+
+// Checkpoints: the first at 32 sweeps (more than the sweeps a decision takes),
+// later ones further apart (one costs about four sweeps of its CTA; replaying
+// from one costs at most an eighth of the sweeps done)
+__device__ __forceinline__ int ckpt_step(int k) { return k < 256 ? 32 : k < 1024 ? 64 : 128; }
+
+// Helper warp: rows from the neighbouring CTA on one side into shared memory.
+template <int C, int R, int WX>
+__device__ __forceinline__ void res_receiver(const ResArgs& a, uint8_t* sm, ResShared& sh, int cta,
+                                             int side)
+{
+    using L = ResLayout<C, R, WX>;
+    constexpr int W = 2 * L::V;  // words per source lane
+    const int lane = threadIdx.x & 31;
+    for (uint32_t t = 1;; ++t) {
+#pragma unroll 1
+        for (int x = 0; x < WX; ++x) {
+            const uint4* p = &a.box->row[cta][side][t & 1u][32 * x + lane];
+            uint4 v[W];
+            int left = kResPolls;
+            for (;;) {
+                bool ok = true;
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    v[i] = ld_box(p + i * 32 * WX);
+                    ok = ok && v[i].y == t && v[i].w == t;
+                }
+                if (__all_sync(0xffffffffu, ok)) break;
+                const uint32_t end = sh.end;
+                if (__any_sync(0xffffffffu, end != 0 && t > end)) return;
+                if (--left <= 0) {
+                    *a.err = 1;
+                    return;
+                }
+            }
+            uint8_t* dst = sm + L::kHalo + (side * 2 + (t & 1u)) * L::kHaloPar + lane * 16;
+#pragma unroll
+            for (int h = 0; h < L::V; ++h)
+                *reinterpret_cast<uint4*>(dst + (x * L::V + h) * 512) =
+                    make_uint4(v[2 * h].x, v[2 * h].z, v[2 * h + 1].x, v[2 * h + 1].z);
+        }
+        __syncwarp();
+        if (lane == 0) bar_arrive(&sh.full[side][t & 1u]);
+    }
+}
+
+// Helper warp: the E rounds of one grid, `first` rounds of other grids before
+// it.  Lane group gi (8 lanes) takes sweep 4q + gi of round q.
+__device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum, ResShared& sh,
+                                           int b, uint32_t first)
+{
+    const int lane = threadIdx.x & 31, gi = lane >> 3, li = lane & 7;
+    const int n = a.n, cta = blockIdx.x, group = cta / n, rank = cta % n;
+    const double inv_cells = 1.0 / ((double)a.nx * (double)a.ny * kSumScale);
+    for (int q = 0;; ++q) {
+        const uint32_t e = first + q, tag = e + 1, slot = e % kResRing;
+        if (!bar_wait(&sh.sums[slot], e / kResRing & 1u, kResSpins)) {
+            *a.err = 1;
+            return;
+        }
+        const float* ws = s_wsum + (e * 4 + gi) % kWsumRing * kResWarps;
+        Pair sum = pair_tree({ws[li] * kSumScale, 0.0f});
+        if (n > 1) {
+            if (li == 0)
+                st_box(&a.box->part[cta][slot][gi], __float_as_uint(sum.h), __float_as_uint(sum.l),
+                       tag);
+            if (rank == 0) {
+                sum = {0.0f, 0.0f};
+                for (int i = li; i < n; i += 8) {
+                    uint4 v;
+                    int left = kResPolls;
+                    do {
+                        v = ld_box(&a.box->part[cta + i][slot][gi]);
+                    } while ((v.y != tag || v.w != tag) && --left > 0);
+                    if (left <= 0) *a.err = 1;
+                    sum = pair_add(sum, {__uint_as_float(v.x), __uint_as_float(v.z)});
+                }
+                __syncwarp();
+                sum = pair_tree(sum);
+            }
+        }
+        int code = 0, ks = 0;
+        if (rank == 0) {
+            // the first lane of each group of eight holds the sum of its sweep
+            const int j = 4 * q + gi;
+            double ej = 0.0;
+            int c = 0;
+            if (li == 0 && (!(sum.h > a.sum_near) || !(sum.h <= 3e38f) || j >= a.cap || a.e_hist)) {
+                ej = ((double)sum.h + (double)sum.l) * inv_cells;
+                if (ej <= a.threshold) c = 1;
+                else if (j >= a.cap || !isfinite(ej)) c = 2;
+            }
+            const uint32_t hit = __ballot_sync(0xffffffffu, c != 0);
+            const int from = hit ? __ffs(hit) - 1 : 31;
+            if (a.e_hist && li == 0 && lane <= from && j < a.hist_len)
+                a.e_hist[(size_t)b * a.hist_len + j] = ej;
+            code = __shfl_sync(0xffffffffu, c, from);
+            ks = 4 * q + (from >> 3);
+            if (lane == from) sh.estar = ej;
+            if (n > 1 && lane == 0)
+                st_box(&a.box->dec[group][slot], (uint32_t)code, (uint32_t)ks, tag);
+        } else {
+            uint4 v;
+            int left = kResPolls;
+            do {
+                v = ld_box(&a.box->dec[group][slot]);
+            } while ((v.y != tag || v.w != tag) && --left > 0);
+            if (left <= 0) {
+                *a.err = 1;
+                v.x = 2;  // leave: the result of this call is void
+                v.z = 0;
+            }
+            code = (int)v.x;
+            ks = (int)v.z;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            if (code != 0) {
+                sh.kstar = ks;
+                sh.code = code;
+                sh.stop = q;
+            }
+            __threadfence_block();
+            sh.rounds = q + 1;
+        }
+        __syncwarp();
+        if (code != 0) return;
+    }
+}
+
+template <int C, int R, int WX>
+__global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const ResArgs a)
+{
+    using L = ResLayout<C, R, WX>;
+    using W = ResWarp<C, R, WX>;
+    extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ ResShared sh;
+    const int n = a.n, cta = blockIdx.x, group = cta / n, rank = cta % n;
+    float* s_wsum = reinterpret_cast<float*>(sm + L::kWsum);
+
+    W w;
+    w.sm = sm;
+    w.lane = threadIdx.x & 31;
+    w.wid = threadIdx.x >> 5;
+    constexpr int kZero = 2 * kResWarps;  // slot of the zero row / column
+    if (threadIdx.x < 32) {
+        const float z[C] = {};
+        for (int p = 0; p < 2; ++p) {
+            w.st_row(L::kRow + p * L::kRowPar + kZero * L::kRowSlot + w.lane * 16, z);
+            if (threadIdx.x < R)
+                *reinterpret_cast<float*>(sm + L::kCol + p * L::kColPar + kZero * R * 4 +
+                                          threadIdx.x * 4) = 0.0f;
+        }
+        if (threadIdx.x < 5) {
+            const CellConst k = make_const(0.0f, (1u << threadIdx.x) - 1u);
+            *reinterpret_cast<float2*>(sm + L::kLut + 8 * threadIdx.x) = make_float2(k.c, k.inv);
+        }
+        if (threadIdx.x == 0) {
+            for (int i = 0; i < 4; ++i) bar_init(&sh.full[i / 2][i % 2], 1);
+            for (int i = 0; i < kResRing; ++i) bar_init(&sh.sums[i], kResWarps);
+            sh.end = 0u;
+        }
+    }
+    __syncthreads();
+
+    if (w.wid >= kResWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kResRegsHelp));
+        if (w.wid == kResWarps) {
+            int b = group;
+            uint32_t first = 0;
+            while (b < a.B) {
+                sync_grid();  // the sweep warps have set the grid up
+                if (!a.fixed || a.gs[b].wild == a.epoch) {
+                    res_rounds(a, s_wsum, sh, b, first);
+                    first += (uint32_t)(sh.stop + kResLag - 1);
+                }
+                sync_grid();  // the grid is done
+                if (a.groups >= a.B) break;
+                sync_grid();
+                b = sh.grid;
+            }
+        } else if (w.wid == kResWarps + 1) {
+            if (rank > 0) res_receiver<C, R, WX>(a, sm, sh, cta, 0);
+        } else if (w.wid == kResWarps + 2) {
+            if (rank < n - 1) res_receiver<C, R, WX>(a, sm, sh, cta, 1);
+        }
+        return;
+    }
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kResRegsSweep));
+
+    w.wx = w.wid % WX;
+    w.wy = w.wid / WX;
+    w.flip = w.wy >= L::WY / 2;
+    const int nx = a.nx, ny = a.ny;
+    const bool vec = (nx & 3) == 0;
+    const bool top = w.wy == 0, bottom = w.wy == L::WY - 1;
+    w.rem = (top && rank > 0) || (bottom && rank < n - 1);
+    {
+        // a row goes into the box of the CTA above (from below) or below (from above)
+        const int peer = top ? cta - 1 : cta + 1;
+        w.tx = w.rem ? &a.box->row[peer][top ? 1 : 0][0][w.wx * 32 + w.lane] : nullptr;
+        const int side = top ? 0 : 1;
+        w.full = sh.full[side];
+        w.in_h = L::kHalo + side * 2 * L::kHaloPar + w.wx * L::kRowSlot + w.lane * 16;
+    }
+    w.t = 0;
+    w.dead = false;
+    const int x0 = (w.wx * 32 + w.lane) * C;
+    const int y0 = (rank * L::WY + w.wy) * R;
+    w.out = x0 >= nx;
+    auto row_of = [&](int r) { return w.flip ? y0 + R - 1 - r : y0 + r; };
+
+    // where the neighbouring rows and columns of this warp are published
+    {
+        auto slot_of = [&](int v, int vy, bool low) {  // warp v, its lower (image) row or upper
+            const bool vf = vy >= L::WY / 2;
+            return 2 * v + (low != vf ? 1 : 0);
+        };
+        const int above = top ? kZero : slot_of(w.wid - WX, w.wy - 1, true);
+        const int below = bottom ? kZero : slot_of(w.wid + WX, w.wy + 1, false);
+        w.in_f = L::kRow + (w.flip ? below : above) * L::kRowSlot + w.lane * 16;
+        w.in_l = L::kRow + (w.flip ? above : below) * L::kRowSlot + w.lane * 16;
+        w.out_r = L::kRow + 2 * w.wid * L::kRowSlot + w.lane * 16;
+        const int cl = w.wx > 0 ? 2 * (w.wid - 1) + 1 : kZero;
+        const int cr = w.wx < WX - 1 ? 2 * (w.wid + 1) : kZero;
+        w.in_c = L::kCol + (w.lane == 31 ? cr : cl) * R * 4;
+        w.out_c = L::kCol + (2 * w.wid + (w.lane == 31 ? 1 : 0)) * R * 4;
+    }
+    // columns an unobstructed inner row has: a wall left of x = 0 and right of nx - 1
+    const bool wall0 = x0 == 0, wall3 = x0 + C == nx;
+    w.c0 = wall0 ? 1.0f : 0.0f;
+    w.c3 = wall3 ? 1.0f : 0.0f;
+    w.invm = w.out ? 0.0f : 0.25f;
+    w.inv0 = w.out ? 0.0f : wall0 ? 1.0f / 3.0f : 0.25f;
+    w.inv3 = w.out ? 0.0f : wall3 ? 1.0f / 3.0f : 0.25f;
+
+    int b = group;
+    uint32_t seq = 0;    // grids this group has begun
+    uint32_t first = 0;  // E rounds of the grids before this one
+    float phi[R][C];
+    while (b < a.B) {
+        ++seq;
+        const size_t gbase = (size_t)b * ny * nx;
+        auto load_cells = [&](const float* src, bool masked, bool v4) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int y = row_of(r);
+#pragma unroll
+                for (int h = 0; h < C; h += 4) {
+                    float f[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                    if (y < ny && src) {
+                        const size_t o = gbase + (size_t)y * nx;
+                        load_row4(src + o, x0 + h, nx, v4, f);
+                        if (masked) {
+                            const uint32_t m4 = load_mask4(a.mask + o, x0 + h, nx, vec);
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                if (((m4 >> (8 * q)) & 15u) == 0u) f[q] = 0.0f;
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) phi[r][h + q] = f[q];
+                }
+            }
+        };
+        auto store_cells = [&](float* dst) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int y = row_of(r);
+                if (y >= ny) continue;
+                float* line = dst + gbase + (size_t)y * nx;
+#pragma unroll
+                for (int h = 0; h < C; h += 4) {
+                    if (vec && x0 + h + 3 < nx) {
+                        *reinterpret_cast<float4*>(line + x0 + h) = make_float4(
+                            phi[r][h], phi[r][h + 1], phi[r][h + 2], phi[r][h + 3]);
+                    } else {
+#pragma unroll
+                        for (int q = h; q < h + 4; ++q)
+                            if (x0 + q < nx) line[x0 + q] = phi[r][q];
+                    }
+                }
+            }
+        };
+
+        // ---- div and the open-face counts on chip, phi_0 in registers
+        w.gen = 0u;
+        w.skip = (1u << (R / 4)) - 1u;
+#pragma unroll 1
+        for (int r = 0; r < R; ++r) {
+            const int y = row_of(r);
+            bool plain = true;
+            uint32_t code = 0;
+#pragma unroll
+            for (int h = 0; h < L::V; ++h) {
+                float dr[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                uint32_t m4 = 0;
+                if (y < ny) {
+                    const size_t o = gbase + (size_t)y * nx;
+                    load_row4(a.div + o, x0 + 4 * h, nx, vec, dr);
+                    m4 = load_mask4(a.mask + o, x0 + 4 * h, nx, vec);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int cnt = __popc((m4 >> (8 * q)) & 15u);
+                    const bool wall = (h == 0 && q == 0 && wall0) ||
+                                      (h == L::V - 1 && q == 3 && wall3);
+                    plain = plain && cnt == (wall ? 3 : 4);
+                    code |= (uint32_t)cnt << (4 * (4 * h + q));
+                }
+                const int slot = ((w.wid * R + r) * L::V + h) * 32 + w.lane;
+                reinterpret_cast<float4*>(sm + L::kDiv)[slot] =
+                    make_float4(dr[0], dr[1], dr[2], dr[3]);
+            }
+            reinterpret_cast<uint32_t*>(sm + L::kCode)[(w.wid * R + r) * 32 + w.lane] = code;
+            if (__any_sync(0xffffffffu, !w.out && y < ny)) w.skip &= ~(1u << (r / 4));
+            if (!__all_sync(0xffffffffu, w.out || plain)) w.gen |= 1u << (r / 4);
+        }
+        load_cells(a.phi0, true, vec && a.phi0_vec);
+        if (threadIdx.x == 0) {
+            sh.act = 0;
+            sh.rounds = 0;
+            sh.stop = -1;
+        }
+        float pending = 0.0f;
+        int kstar = a.cap, dec = 2;
+        double estar = 0.0;
+        w.publish(phi);
+        sync_grid();
+
+        const bool with_e = !a.fixed || a.gs[b].wild == a.epoch;
+        int base = 0;  // the iterate that a replay would start from
+        const float* from = a.phi0;
+        if (with_e) {
+            // phi at the cap: not where a checkpoint it may still need lies
+            float* cap_buf = a.cap < 64 ? a.ck[1] : a.phi;
+            int last = 0, before = 0, cb = 1;  // latest checkpoints, buffer of the latest
+            // four sweeps at a time; round q needs the sums of sweeps 4q .. 4q+3,
+            // the last stored during sweep 4q + 4
+            int k = 0;
+            for (;; k += 4) {
+                if (sh.act != 0) break;
+                if (k == last + ckpt_step(last) && k <= a.cap) {
+                    cb ^= 1;
+                    store_cells(a.ck[cb]);
+                    before = last;
+                    last = k;
+                }
+#pragma unroll 1
+                for (int i = 0; i < 4; ++i) {
+                    if (i == 2 && threadIdx.x == 0 && k + 4 >= 4 * kResLag) {
+                        // the decision of round k / 4 + 1 - kResLag: long there
+                        const int q = k / 4 + 1 - kResLag;
+                        int left = kResSpins;
+                        while (sh.rounds <= q && --left > 0) {
+                        }
+                        if (left <= 0) {
+                            *a.err = 1;
+                            sh.kstar = 0;
+                            sh.code = 2;
+                            sh.estar = 0.0;
+                            sh.stop = q;
+                        }
+                        __threadfence_block();
+                        if (sh.stop == q) sh.act = 1;
+                    }
+                    float* wsum = s_wsum + ((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
+                                  w.wid;
+                    if (k + i <= a.cap) {
+                        if (k + i == a.cap) store_cells(cap_buf);
+                        w.template update<true>(phi, pending, wsum, a.err);
+                    } else if (k + i - 1 == a.cap) {
+                        // past the cap only its sum is left to do
+                        float s = pending;
+#pragma unroll
+                        for (int off = 16; off > 0; off >>= 1)
+                            s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
+                        if (w.lane == 0) *wsum = s;
+                    }
+                    if (i == 0 && k > 0 && w.lane == 0)
+                        bar_arrive(&sh.sums[(first + k / 4 - 1) % kResRing]);
+                    sync_sweepers();
+                }
+            }
+            kstar = sh.kstar;
+            dec = sh.code;
+            estar = sh.estar;
+            first += (uint32_t)(k / 4 - 1);
+            w.drain(a.err);
+            if (kstar == a.cap && cap_buf != a.phi) {
+                // each thread its own cells
+                load_cells(cap_buf, false, vec);
+                store_cells(a.phi);
+            }
+            base = kstar >= last ? last : before;
+            from = base == 0 ? a.phi0 : base == last ? a.ck[cb] : a.ck[cb ^ 1];
+        }
+        if (!with_e || kstar != a.cap) {
+            // ---- from phi_0 or the checkpoint at or below k* to phi_{k*}
+            if (with_e) {
+                load_cells(from, base == 0, vec && (base != 0 || a.phi0_vec));
+                sync_sweepers();
+                w.publish(phi);
+                sync_sweepers();
+            }
+            for (int j = base; j < kstar; ++j) {
+                w.template update<false>(phi, pending, nullptr, a.err);
+                sync_sweepers();
+            }
+            store_cells(a.phi);
+            w.drain(a.err);
+        }
+        if (threadIdx.x == 0 && rank == 0) {
+            GridState* gs = a.gs + b;
+            gs->active = 0;
+            gs->kstar = kstar;
+            gs->k0_stop = kstar;
+            gs->replay = 0;
+            gs->src = 0;
+            gs->final_buf = 0;
+            gs->converged = dec == 1 ? 1 : 0;
+            gs->e_stop = estar;
+        }
+        // ---- next grid: in turn when every grid takes the same sweeps, else
+        // whichever is left (rank 0 asks, the group follows)
+        sync_grid();
+        if (a.groups >= a.B) break;
+        if (threadIdx.x == 0) {
+            uint4* nb = &a.box->next[group][seq & 1u];
+            if (a.fixed) {
+                sh.grid = b + a.groups;
+            } else if (rank == 0) {
+                sh.grid = a.groups + (int)atomicAdd(&a.box->queue, 1u);
+                if (n > 1) st_box(nb, (uint32_t)sh.grid, 0u, seq);
+            } else {
+                uint4 v;
+                int left = kResPolls;
+                do {
+                    v = ld_box(nb);
+                } while (v.y != seq && --left > 0);
+                if (left <= 0) {
+                    *a.err = 1;
+                    v.x = (uint32_t)a.B;
+                }
+                sh.grid = (int)v.x;
+            }
+        }
+        sync_grid();
+        b = sh.grid;
+    }
+    if (threadIdx.x == 0) sh.end = w.t;
+}
+
+// An instance: its function, dynamic shared memory and strip height.
+struct ResKernel {
+    const void* fn;
+    int smem;
+    int rows;  // of one CTA
+};
+
+template <int C, int R, int WX>
+ResKernel res_kernel()
+{
+    using L = ResLayout<C, R, WX>;
+    return {(const void*)sweep_resident_kernel<C, R, WX>, L::kBytes, L::WY * R};
+}
+
+// by width of the grid, with `rows` rows per thread (4, 8 or 16)
+ResKernel res_kernel_128(int rows);
+ResKernel res_kernel_256(int rows);
+ResKernel res_kernel_512(int rows);
+
+}  // namespace hp
