@@ -84,10 +84,10 @@ typedef struct {
  *                  2 = temporally blocked (T
  *                  sweeps per launch, replay to the exact stop; 4 rows per
  *                  thread), 3 = temporally blocked with 2 rows per thread
- *                  (twice the warps), 4 = grid-resident: strips of whole
- *                  rows on up to all SMs of the device keep a grid on chip
- *                  for all sweeps (grids up to 512 cells wide), falling back
- *                  to 2 for wider grids.  All give the same iterates bit for
+ *                  (twice the warps), 4 = grid-resident: strips of a grid,
+ *                  one on each SM, keep it on chip for all sweeps, falling
+ *                  back to 2 for grids that the SMs do not hold (somewhat
+ *                  above 2048 x 2048).  All give the same iterates bit for
  *                  bit; the FP64 E_k may differ in the last bits between
  *                  kernels (their partial sums are grouped differently).
  *   open_top       1 = the top boundary (the v faces of row 0) is open to an

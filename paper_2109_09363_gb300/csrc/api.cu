@@ -140,6 +140,7 @@ void hp_ctx_destroy(hp_ctx* c)
     cudaFree(c->gs);
     cudaFree(c->ls);
     cudaFree(c->box);
+    cudaFree(c->cols);
     cudaFree(c->wait_err);
     if (c->host_flag) cudaFreeHost(c->host_flag);
     if (prev >= 0) cudaSetDevice(prev);
@@ -187,6 +188,8 @@ hp_status hp_ctx_create(hp_ctx** out, hp_shape mx, int device)
         (rc = dalloc(&c->gs, (size_t)mx.batch, &c->guards)) != HP_OK ||
         (rc = dalloc(&c->ls, 1, &c->guards)) != HP_OK ||
         (rc = dalloc((uint8_t**)&c->box, resident_box_bytes(), &c->guards)) != HP_OK ||
+        (mx.nx > 512 &&
+         (rc = dalloc((uint8_t**)&c->cols, resident_columns_bytes(), &c->guards)) != HP_OK) ||
         (rc = dalloc(&c->wait_err, 1, &c->guards)) != HP_OK) {
         hp_ctx_destroy(c);
         return rc;

@@ -121,6 +121,7 @@ struct hp_ctx {
     hp::LoopState* ls;
     float* ckpt;         // [max_cells] checkpoint buffer of the resident sweep kernel
     void* box;           // exchange area of the resident sweep kernel (ResBox)
+    void* cols;          // that of copied columns (ResColumns), null for max nx <= 512
     int32_t* wait_err;   // set by a bounded wait of that kernel that gave up
     uint32_t epoch;      // its launches
     int32_t* host_flag;  // pinned
@@ -217,6 +218,7 @@ __device__ __forceinline__ uint32_t load_mask4(const uint8_t* __restrict__ row, 
 
 void set_cuda_error(cudaError_t e);
 size_t resident_box_bytes();
+size_t resident_columns_bytes();
 int resident_capacity(hp_ctx* ctx, hp_shape s);
 hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bool fixed,
                           const float* phi0, double* e_hist, int hist_len, cudaStream_t st,

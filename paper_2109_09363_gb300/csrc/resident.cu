@@ -8,13 +8,16 @@ namespace {
 
 ResKernel res_kernel(int width, int R)
 {
-    return width == 128 ? res_kernel_128(R) : width == 256 ? res_kernel_256(R) : res_kernel_512(R);
+    return width == 128   ? res_kernel_128(R)
+           : width == 256 ? res_kernel_256(R)
+           : width == 512 ? res_kernel_512(R)
+                          : res_kernel_wide(R);
 }
 
 // How a grid is split: columns of warps, rows per thread, CTAs per grid and
 // grids at once.
 struct ResPlan {
-    int width, R, n, groups;
+    int width, R, n, ntx, groups;
 };
 
 // CTAs of a cooperative launch that fit on the device: one per SM (every
@@ -22,29 +25,34 @@ struct ResPlan {
 int res_ctas(const hp_ctx* ctx) { return ctx->num_sms < kResMaxCtas ? ctx->num_sms : kResMaxCtas; }
 
 // The split with the least time: waves of groups x time per sweep of a strip,
-// measured (16 x 512^2, 8 x 256^2 and 152 x 128^2 grids with obstacles).  More
+// measured (16 x 512^2, 8 x 256^2, 152 x 128^2 and, for columns, 2048^2 grids with
+// obstacles).  More
 // rows per thread make a longer sweep with less of it lost to the exchange,
 // fewer rows spread a grid over more SMs: 16 x 512^2 takes 5.0, 3.8 and 5.5 us
 // per sweep with 4, 8 and 16 rows (four, two waves and one), one 512^2 grid
 // 1.27, 1.83 and 3.2 us.
 bool res_plan(const hp_ctx* ctx, hp_shape s, ResPlan* best)
 {
-    if (s.nx > 512) return false;
-    const int width = s.nx <= 128 ? 128 : s.nx <= 256 ? 256 : 512;
+    // wider than 512 cells: columns of 240, eight copied on each side
+    const int width = s.nx <= 128 ? 128 : s.nx <= 256 ? 256 : s.nx <= 512 ? 512 : 1024;
+    const int own = 256 - 2 * kResGhost;
+    const int ntx = width == 1024 ? (s.nx + own - 1) / own : 1;
     // us per sweep of a strip with E, on grids with obstacles, R = 4, 8, 16
-    static const double us[3][3] = {{0.72, 1.0, 1.78}, {1.12, 1.84, 3.3}, {1.27, 1.85, 4.4}};
+    static const double us[4][3] = {
+        {0.72, 1.0, 1.78}, {1.12, 1.84, 3.3}, {1.27, 1.85, 4.4}, {0.0, 2.03, 3.82}};
     const int ctas = res_ctas(ctx);
     double least = 0.0;
     bool found = false;
     for (int R : {4, 8, 16}) {
-        const int rows = res_kernel(width, R).rows, n = (s.ny + rows - 1) / rows;
+        if (R == 4 && width == 1024) continue;
+        const int rows = res_kernel(width, R).rows, n = (s.ny + rows - 1) / rows * ntx;
         if (n > ctas) continue;
         const int groups = ctas / n < s.batch ? ctas / n : s.batch;
         const int waves = (s.batch + groups - 1) / groups;
-        const double t = waves * us[width / 256][R / 8];
+        const double t = waves * us[width == 128 ? 0 : width == 256 ? 1 : width == 512 ? 2 : 3][R / 8];
         if (!found || t < least) {
             least = t;
-            *best = {width, R, n, groups};
+            *best = {width, R, n, ntx, groups};
             found = true;
         }
     }
@@ -54,7 +62,8 @@ bool res_plan(const hp_ctx* ctx, hp_shape s, ResPlan* best)
 // Per-grid state, the exchange area of `ctas` CTAs in groups (n > 1), and, for
 // a fixed number of sweeps, which grids hold values so large that a sum of
 // residuals could overflow: those stop at the first non-finite E.
-__global__ void resident_prep_kernel(GridState* gs, ResBox* box, int B, int ctas, int n,
+__global__ void resident_prep_kernel(GridState* gs, ResBox* box, ResColumns* cols, int B, int ctas,
+                                     int n,
                                      const float* __restrict__ div,
                                      const float* __restrict__ phi0, size_t cells, uint32_t epoch,
                                      int scan)
@@ -73,6 +82,9 @@ __global__ void resident_prep_kernel(GridState* gs, ResBox* box, int B, int ctas
         for (size_t i = id; i < (size_t)ctas * kResRing; i += step) dec[i] = z;
         uint4* next = &box->next[0][0];
         for (size_t i = id; i < (size_t)ctas * 2; i += step) next[i] = z;
+        uint4* col = cols ? &cols->w[0][0][0][0][0][0] : nullptr;
+        if (col)
+            for (size_t i = id; i < (size_t)ctas * 2 * 2 * kResWarps * 2 * 32; i += step) col[i] = z;
     }
     if (scan) {
         constexpr float kTame = 1e20f;  // |phi| grows by max |div| per sweep at most
@@ -86,6 +98,7 @@ __global__ void resident_prep_kernel(GridState* gs, ResBox* box, int B, int ctas
 }  // namespace
 
 size_t resident_box_bytes() { return sizeof(ResBox); }
+size_t resident_columns_bytes() { return sizeof(ResColumns); }
 
 // Grids of shape s held on chip at once; 0 above 512 x 512 cells.
 int resident_capacity(hp_ctx* ctx, hp_shape s)
@@ -120,6 +133,8 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     a.mask = ctx->mask;
     a.gs = ctx->gs;
     a.box = (ResBox*)ctx->box;
+    a.cols = p.ntx > 1 ? (ResColumns*)ctx->cols : nullptr;
+    a.ntx = p.ntx;
     a.err = ctx->wait_err;
     a.e_hist = e_hist;
     a.hist_len = hist_len;
@@ -138,7 +153,7 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     const size_t work = a.fixed ? cells * s.batch / 8 : p.n > 1 ? (size_t)ctas * 1024 : s.batch;
     const size_t want = work / 256 + 1, most = 8 * (size_t)ctx->num_sms;
     resident_prep_kernel<<<(unsigned)(want < most ? want : most), 256, 0, st>>>(
-        ctx->gs, a.box, s.batch, ctas, p.n, ctx->div, phi0, cells, a.epoch, a.fixed);
+        ctx->gs, a.box, a.cols, s.batch, ctas, p.n, ctx->div, phi0, cells, a.epoch, a.fixed);
     hp_status rc = check_launch();
     if (rc != HP_OK) return rc;
     cudaLaunchConfig_t cfg = {};

@@ -23,6 +23,12 @@
 //     zero), the others look 4 - n and 1/n up by the cell's bits.
 // The only barrier of a sweep is the CTA's own.
 //
+// Grids wider than 512 cells are also cut into columns of 240 cells: a CTA then
+// holds 256 columns, the outer 8 on each side copies of its neighbours' cells.
+// A copy is good for one column less after every sweep, so they are fetched
+// anew every 8 sweeps (through the L2 as well), which costs two exposed round
+// trips in 8 sweeps instead of one more exchange in each.
+//
 // E_k: FP32 |r| per thread and warp, then sums of float pairs (TwoSum, 48
 // bits; an FP64 addition of a warp occupies its scheduler's FP64 unit for 64
 // cycles here, and four dependent ones per round cost 0.6 us a sweep) per CTA
@@ -76,6 +82,15 @@ struct ResBox {
     uint32_t queue;                        // grids handed out beyond the first of each group
 };
 
+// Columns of a strip that are copies, on each side, and sweeps they last.
+constexpr int kResGhost = 8;
+
+// Columns from the CTAs beside (grids wider than 512 cells): [receiver][side:
+// from the left, from the right][parity][warp][word][lane]
+struct ResColumns {
+    uint4 w[kResMaxCtas][2][2][kResWarps][2][32];
+};
+
 struct ResArgs {
     const float* phi0;  // phi_0 of the caller (cells without an open face ignored), null = 0
     float* phi;         // phi_{k*} out (may be phi0)
@@ -84,11 +99,12 @@ struct ResArgs {
     const uint8_t* mask;
     GridState* gs;
     ResBox* box;
+    ResColumns* cols;   // null unless ntx > 1
     int32_t* err;       // set to 1 when a wait gave up
     double* e_hist;     // [B][hist_len] or null
     int32_t hist_len;
     int32_t B, ny, nx;
-    int32_t n;          // CTAs per grid
+    int32_t n, ntx;     // CTAs per grid, side by side
     int32_t groups;
     int32_t cap;
     int32_t phi0_vec;   // phi0 allows 16-byte loads
@@ -116,7 +132,9 @@ struct ResLayout {
     static constexpr int kHaloPar = WX * kRowSlot;
     static constexpr int kLut = kHalo + 4 * kHaloPar;                    // [5] float2
     static constexpr int kWsum = kLut + 64;                              // [16][8] float
-    static constexpr int kBytes = kWsum + kWsumRing * kResWarps * 4;
+    // copied columns in transit: [warp][2 sides][R][8] float
+    static constexpr int kGhost = kWsum + kWsumRing * kResWarps * 4;
+    static constexpr int kBytes = kGhost + kResWarps * 2 * R * kResGhost * 4;
     static_assert(R % 4 == 0 && C % 4 == 0, "rows and columns go out four values at a time");
     static_assert(kBytes <= 227 * 1024 - 64, "shared memory of one CTA");
 };
@@ -217,7 +235,8 @@ struct ResWarp {
     int lane, wid, wx, wy;
     bool flip;        // register row r is image row y0 + R - 1 - r
     bool rem;         // the row beside register row 0 comes from another CTA
-    bool out;         // this lane lies right of the grid
+    bool out;         // this lane lies outside the grid
+    bool mute;        // its residuals are not this CTA's to sum
     uint32_t gen;     // bit g: some cell of rows 4g..4g+3 differs from its column's default
     uint32_t skip;    // bit g: rows 4g..4g+3 lie outside the grid
     float c0, inv0, invm, inv3, c3;  // column defaults (first, inner and last cell; inner c = 0)
@@ -427,7 +446,7 @@ struct ResWarp {
         ++t;
         if (WITH_E) {
             if (lane == 0) *wsum = s;
-            pending = out ? 0.0f
+            pending = mute ? 0.0f
                           : __fadd_rn(__fadd_rn(acc[0], acc[1]), __fadd_rn(acc[2], acc[3]));
         }
     }
@@ -517,14 +536,24 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
                        tag);
             if (rank == 0) {
                 sum = {0.0f, 0.0f};
-                for (int i = li; i < n; i += 8) {
-                    uint4 v;
+                for (int i = li; i < n; i += 32) {  // four loads in flight
+                    uint4 v[4];
                     int left = kResPolls;
+                    bool ok;
                     do {
-                        v = ld_box(&a.box->part[cta + i][slot][gi]);
-                    } while ((v.y != tag || v.w != tag) && --left > 0);
+                        ok = true;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int c = i + 8 * u < n ? i + 8 * u : i;
+                            v[u] = ld_box(&a.box->part[cta + c][slot][gi]);
+                            ok = ok && v[u].y == tag && v[u].w == tag;
+                        }
+                    } while (!ok && --left > 0);
                     if (left <= 0) *a.err = 1;
-                    sum = pair_add(sum, {__uint_as_float(v.x), __uint_as_float(v.z)});
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (i + 8 * u < n)
+                            sum = pair_add(sum, {__uint_as_float(v[u].x), __uint_as_float(v[u].z)});
                 }
                 __syncwarp();
                 sum = pair_tree(sum);
@@ -579,14 +608,90 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
     }
 }
 
-template <int C, int R, int WX>
+// The copied columns of phi from the CTAs beside (left, right: there is one),
+// message m: each warp sends its first and last own columns and waits for its
+// neighbours' (the same warp of those CTAs, so message m + 2 cannot overtake
+// message m).
+template <int R, int WX>
+__device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float (&phi)[R][8],
+                                            int cta, int wid, int lane, bool left, bool right,
+                                            uint32_t m, bool& dead)
+{
+    using L = ResLayout<8, R, WX>;
+    constexpr int W = R / 8;  // words per lane and side
+    float* stage = reinterpret_cast<float*>(sm + L::kGhost) + wid * 2 * R * kResGhost;
+    __syncwarp();
+    if (lane == 1 || lane == 30) {
+        float4* dst = reinterpret_cast<float4*>(stage + (lane == 1 ? 0 : R * kResGhost));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            dst[2 * r] = make_float4(phi[r][0], phi[r][1], phi[r][2], phi[r][3]);
+            dst[2 * r + 1] = make_float4(phi[r][4], phi[r][5], phi[r][6], phi[r][7]);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        if (side ? !right : !left) continue;
+        uint4* box = a.cols->w[side ? cta + 1 : cta - 1][side ^ 1][m & 1u][wid][0];
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const float2 v =
+                *reinterpret_cast<const float2*>(stage + side * R * kResGhost + (i * 32 + lane) * 2);
+            st_box(box + i * 32 + lane, __float_as_uint(v.x), __float_as_uint(v.y), m);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        if (side ? !right : !left) continue;
+        const uint4* box = a.cols->w[cta][side][m & 1u][wid][0];
+        uint4 v[W];
+        int polls = dead ? 1 : kResPolls;
+        for (;;) {
+            bool ok = true;
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                v[i] = ld_box(box + i * 32 + lane);
+                ok = ok && v[i].y == m && v[i].w == m;
+            }
+            if (__all_sync(0xffffffffu, ok)) break;
+            if (--polls <= 0) {
+                dead = true;
+                *a.err = 1;
+                break;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            *reinterpret_cast<float2*>(stage + side * R * kResGhost + (i * 32 + lane) * 2) =
+                make_float2(__uint_as_float(v[i].x), __uint_as_float(v[i].z));
+    }
+    __syncwarp();
+    if ((lane == 0 && left) || (lane == 31 && right)) {
+        const float4* src = reinterpret_cast<const float4*>(stage + (lane == 0 ? 0 : R * kResGhost));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 u = src[2 * r], v = src[2 * r + 1];
+            phi[r][0] = u.x; phi[r][1] = u.y; phi[r][2] = u.z; phi[r][3] = u.w;
+            phi[r][4] = v.x; phi[r][5] = v.y; phi[r][6] = v.z; phi[r][7] = v.w;
+        }
+    }
+    __syncwarp();
+}
+
+// WIDE: the grid is cut into columns too
+template <int C, int R, int WX, bool WIDE>
 __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const ResArgs a)
 {
     using L = ResLayout<C, R, WX>;
     using W = ResWarp<C, R, WX>;
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ ResShared sh;
+    static_assert(!WIDE || (C == kResGhost && WX == 1), "one lane of copies on each side");
     const int n = a.n, cta = blockIdx.x, group = cta / n, rank = cta % n;
+    // strips above one another are ntx CTAs apart
+    const int ntx = WIDE ? a.ntx : 1, ty = rank / ntx, tx = rank % ntx, nty = n / ntx;
     float* s_wsum = reinterpret_cast<float*>(sm + L::kWsum);
 
     W w;
@@ -631,9 +736,9 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                 b = sh.grid;
             }
         } else if (w.wid == kResWarps + 1) {
-            if (rank > 0) res_receiver<C, R, WX>(a, sm, sh, cta, 0);
+            if (ty > 0) res_receiver<C, R, WX>(a, sm, sh, cta, 0);
         } else if (w.wid == kResWarps + 2) {
-            if (rank < n - 1) res_receiver<C, R, WX>(a, sm, sh, cta, 1);
+            if (ty < nty - 1) res_receiver<C, R, WX>(a, sm, sh, cta, 1);
         }
         return;
     }
@@ -645,10 +750,10 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
     const int nx = a.nx, ny = a.ny;
     const bool vec = (nx & 3) == 0;
     const bool top = w.wy == 0, bottom = w.wy == L::WY - 1;
-    w.rem = (top && rank > 0) || (bottom && rank < n - 1);
+    w.rem = (top && ty > 0) || (bottom && ty < nty - 1);
     {
         // a row goes into the box of the CTA above (from below) or below (from above)
-        const int peer = top ? cta - 1 : cta + 1;
+        const int peer = top ? cta - ntx : cta + ntx;
         w.tx = w.rem ? &a.box->row[peer][top ? 1 : 0][0][w.wx * 32 + w.lane] : nullptr;
         const int side = top ? 0 : 1;
         w.full = sh.full[side];
@@ -656,9 +761,12 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
     }
     w.t = 0;
     w.dead = false;
-    const int x0 = (w.wx * 32 + w.lane) * C;
-    const int y0 = (rank * L::WY + w.wy) * R;
-    w.out = x0 >= nx;
+    const bool left = WIDE && tx > 0, right = WIDE && tx < ntx - 1;
+    const int x0 = (WIDE ? tx * (32 * C - 2 * kResGhost) - kResGhost : 0) + (w.wx * 32 + w.lane) * C;
+    const int y0 = (ty * L::WY + w.wy) * R;
+    const bool copy = WIDE && (w.lane == 0 || w.lane == 31);
+    w.out = x0 < 0 || x0 >= nx;
+    w.mute = w.out || copy;
     auto row_of = [&](int r) { return w.flip ? y0 + R - 1 - r : y0 + r; };
 
     // where the neighbouring rows and columns of this warp are published
@@ -688,6 +796,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
     int b = group;
     uint32_t seq = 0;    // grids this group has begun
     uint32_t first = 0;  // E rounds of the grids before this one
+    uint32_t fetched = 0;  // messages with copied columns
     float phi[R][C];
     while (b < a.B) {
         ++seq;
@@ -718,7 +827,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int y = row_of(r);
-                if (y >= ny) continue;
+                if (y >= ny || copy) continue;
                 float* line = dst + gbase + (size_t)y * nx;
 #pragma unroll
                 for (int h = 0; h < C; h += 4) {
@@ -734,6 +843,15 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             }
         };
 
+        // the copied columns anew; the boundary rows go out again with them
+        auto refresh = [&]() {
+            if constexpr (WIDE) {
+                ++fetched;
+                res_columns<R, WX>(a, sm, phi, cta, w.wid, w.lane, left, right, fetched, w.dead);
+                w.publish(phi);
+                sync_sweepers();
+            }
+        };
         // ---- div and the open-face counts on chip, phi_0 in registers
         w.gen = 0u;
         w.skip = (1u << (R / 4)) - 1u;
@@ -797,6 +915,10 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     before = last;
                     last = k;
                 }
+                if (WIDE && k > 0 && k % kResGhost == 0 && k <= a.cap) {
+                    w.drain(a.err);
+                    refresh();
+                }
 #pragma unroll 1
                 for (int i = 0; i < 4; ++i) {
                     if (i == 2 && threadIdx.x == 0 && k + 4 >= 4 * kResLag) {
@@ -851,10 +973,18 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             if (with_e) {
                 load_cells(from, base == 0, vec && (base != 0 || a.phi0_vec));
                 sync_sweepers();
-                w.publish(phi);
-                sync_sweepers();
+                if (WIDE && base > 0) {
+                    refresh();
+                } else {
+                    w.publish(phi);
+                    sync_sweepers();
+                }
             }
             for (int j = base; j < kstar; ++j) {
+                if (WIDE && j > base && j % kResGhost == 0) {
+                    w.drain(a.err);
+                    refresh();
+                }
                 w.template update<false>(phi, pending, nullptr, a.err);
                 sync_sweepers();
             }
@@ -909,16 +1039,17 @@ struct ResKernel {
     int rows;  // of one CTA
 };
 
-template <int C, int R, int WX>
+template <int C, int R, int WX, bool WIDE = false>
 ResKernel res_kernel()
 {
     using L = ResLayout<C, R, WX>;
-    return {(const void*)sweep_resident_kernel<C, R, WX>, L::kBytes, L::WY * R};
+    return {(const void*)sweep_resident_kernel<C, R, WX, WIDE>, L::kBytes, L::WY * R};
 }
 
 // by width of the grid, with `rows` rows per thread (4, 8 or 16)
 ResKernel res_kernel_128(int rows);
 ResKernel res_kernel_256(int rows);
 ResKernel res_kernel_512(int rows);
+ResKernel res_kernel_wide(int rows);  // 8 or 16 rows; columns of 240 cells
 
 }  // namespace hp
