@@ -14,6 +14,8 @@
 // commits them to an mbarrier, and the 128 threads read their row back with
 // tcgen05.ld.  This gather form serves widths below 32; wider images use the
 // warp-specialised row walk further down.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -46,6 +48,15 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return d;
 }
 
+// The same for a K-major operand whose rows (pitch 32, 64 or 128 bytes) are
+// swizzled as a TMA tile of that inner width: groups of eight rows are
+// contiguous; K steps and whole-row shifts move the start address.
+__device__ __forceinline__ uint64_t smem_desc_swizzled(uint32_t addr, int pitch)
+{
+    const uint64_t mode = pitch == 128 ? 2 : pitch == 64 ? 4 : 6;
+    return smem_desc(addr, 16, 8 * pitch) | mode << 61;
+}
+
 // Instruction descriptor, kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, N = n, M = m.
 __host__ __device__ constexpr uint32_t mma_idesc(int m, int n)
@@ -61,6 +72,30 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+// The same issued by one lane of a warp whose lanes all run the call with the
+// same arguments: in uniform control flow the descriptors stay in uniform
+// registers.  (From a branch of one lane every MMA first moved its operands
+// there, 107-125 cycles per MMA, at N = 96 twice what the MMA takes.)
+__device__ __forceinline__ void mma_bf16_warp(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                              uint32_t idesc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, one;\n\telect.sync _|one, 0xffffffff;\n\t"
+        "setp.eq.b32 p, 0, 0;\n\t"
+        "@one tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_commit_warp(uint32_t mbar)
+{
+    asm volatile(
+        "{\n\t.reg .pred one;\n\telect.sync _|one, 0xffffffff;\n\t"
+        "@one tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::
+            "r"(mbar)
+        : "memory");
 }
 
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase)
@@ -314,7 +349,7 @@ constexpr int kWsSlots = 6;
 // width 64 0.171 ms (gather 0.434 ms), width 32 0.088 ms (gather 0.119 ms).
 constexpr int kWsMinWidth = 32;
 constexpr int kAccSlots = 8;
-constexpr int kWsThreads = 192;
+constexpr int kWsThreads = 224;
 constexpr uint32_t kWsSpinLimit = 1u << 22;
 
 // CTAs per SM: the edge layers of a branch (16 -> 32 and the 32 -> 1 layer
@@ -333,7 +368,9 @@ constexpr int ws_ctas_per_sm()
 template <int CIN, int COUT, bool OUT1 = false>
 struct WsSmem {
     static constexpr int kChunks = CIN / 8;
-    static constexpr int kSlotBytes = kChunks * kHaloPx * 16;
+    static constexpr int kPitch = 2 * CIN;  // bytes of a pixel
+    static constexpr int kRowBytes = kHaloPx * kPitch;
+    static constexpr int kSlotBytes = (kRowBytes + 1023) / 1024 * 1024;
     static constexpr int kRingBytes = kWsSlots * kSlotBytes;
     static constexpr int kBBytes = 9 * kChunks * COUT * 16;
     // per epilogue warp: its 32 output pixels in BF16, 16-byte chunks XOR-swizzled
@@ -359,6 +396,22 @@ __device__ __forceinline__ bool mbar_wait_ws(uint32_t mbar, uint32_t parity,
                                              const volatile int* abort_flag,
                                              uint32_t limit = kWsSpinLimit)
 {
+    // a limit of the caller's counts plain looks; the compiled one counts
+    // waits that the hardware may suspend for a while
+    if (limit != kWsSpinLimit) {
+        for (uint32_t it = 0; it < limit; ++it) {
+            uint32_t done;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}\n"
+                : "=r"(done)
+                : "r"(mbar), "r"(parity)
+                : "memory");
+            if (done) return true;
+            if ((it & 1023u) == 1023u && *abort_flag) return false;
+        }
+        return false;
+    }
     for (uint32_t it = 0; it < limit; ++it) {
         uint32_t done;
         asm volatile(
@@ -470,6 +523,11 @@ __device__ __forceinline__ uint32_t relu_mask2(uint32_t v, uint32_t a)
     return v & m;
 }
 
+template <bool F>
+struct Flag {
+    static constexpr bool value = F;
+};
+
 struct WsItem {
     int b, x0, y0, y1;
 };
@@ -502,10 +560,11 @@ __device__ __forceinline__ uint32_t idesc_for_rows(int n_out, int cout)
 // derivative of the layer that produced act; act may be null).
 template <int CIN, int COUT, bool OUT1, bool DGRAD = false>
 __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()))
-    conv3x3_tc_ws_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w,
+    conv3x3_tc_ws_kernel(const uint4* __restrict__ w,
                          const float* __restrict__ bias, void* __restrict__ yout, int H, int W,
                          int segs, int nbands, int band, int items, int relu, int* err,
-                         uint32_t wait_limit, const uint4* __restrict__ act = nullptr)
+                         uint32_t wait_limit, const uint4* __restrict__ act,
+                         const __grid_constant__ CUtensorMap xmap)
 {
     using S = WsSmem<CIN, COUT, OUT1>;
     // polls of each pipeline wait before it gives up (0: the compiled limit);
@@ -517,6 +576,7 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
     uint8_t* ring = smem;
     uint8_t* sB = smem + S::kRingBytes;
     __shared__ __align__(8) uint64_t full_bar[kWsSlots];
+    __shared__ __align__(8) uint64_t raw_bar[kWsSlots];  // copied, borders not replicated yet
     __shared__ __align__(8) uint64_t empty_bar[kWsSlots];
     __shared__ __align__(8) uint64_t outf_bar[kAccSlots];
     __shared__ __align__(8) uint64_t free_bar[kAccSlots];
@@ -537,7 +597,9 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
     if (tid == 0) {
         for (int s = 0; s < kWsSlots; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full_bar[s])),
-                         "r"(32u));
+                         "r"(1u));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&raw_bar[s])),
+                         "r"(1u));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty_bar[s])),
                          "r"(1u));
         }
@@ -587,57 +649,96 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     bool ok = true;
 
+    // a tile whose halo crosses the image's left or right border gets the
+    // replicated pixel there by hand (the copy fills it with zeros)
+    auto at_border = [&](const WsItem& it) {
+        return !DGRAD && (it.x0 == 0 || it.x0 + kHaloPx - 1 > W);
+    };
     if (warp == 5) {
         // ---------------------------------------------------------- producer
-        // lane: channel chunk ch of pixels p0, p0 + kPass, ...; a warp copies
-        // kPass whole pixels (512 contiguous bytes) per instruction
-        constexpr int kPass = 32 / NCH;
-        const int ch = lane % NCH, p0 = lane / NCH;
-        uint32_t jg = 0;
-        for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-            const WsItem it = ws_item(wi, segs, nbands, band, H);
-            const bool interior = it.x0 >= 1 && it.x0 + kHaloPx - 1 <= W;
-            for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jg) {
-                const uint32_t s = jg % kWsSlots, u = jg / kWsSlots;
-                // the lanes take one decision (no lane runs ahead of the others)
-                if (u > 0)
-                    ok = __all_sync(0xffffffffu,
-                                    mbar_wait_ws(smem_u32(&empty_bar[s]), (u - 1) & 1u, &s_abort,
-                                                 lim));
-                if (!ok) break;
-                const int sr = min(max(r, 0), H - 1);
-                const uint32_t dst = smem_u32(ring + s * S::kSlotBytes) + (uint32_t)(ch * kHaloPx * 16);
-                const uint4* src_row = x + ((size_t)it.b * H + sr) * W * NCH + ch;
-                if constexpr (DGRAD) {
-                    // zero outside the image
-                    const bool row_in = r >= 0 && r < H;
-                    for (int px = p0; px < kHaloPx; px += kPass) {
-                        const int gx = it.x0 - 1 + px;
-                        const int sx = min(max(gx, 0), W - 1);
-                        cp_async16_zfill(dst + (uint32_t)(px * 16), src_row + (size_t)sx * NCH,
-                                         row_in && gx >= 0 && gx < W);
-                    }
-                } else if (interior) {
-                    const uint4* src = src_row + (size_t)(it.x0 - 1 + p0) * NCH;
-#pragma unroll 4
-                    for (int px = p0; px < kHaloPx; px += kPass, src += kPass * NCH)
-                        cp_async16(dst + (uint32_t)(px * 16), src);
-                } else {
-                    for (int px = p0; px < kHaloPx; px += kPass) {
-                        const int sx = min(max(it.x0 - 1 + px, 0), W - 1);
-                        cp_async16(dst + (uint32_t)(px * 16), src_row + (size_t)sx * NCH);
-                    }
+        if (lane == 0) {
+            uint32_t jg = 0, raw = 0;  // raw: parity of the next phase of raw_bar[s]
+            uint32_t last_raw = 0;     // bit s: the last copy into slot s signalled raw_bar
+            for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
+                const WsItem it = ws_item(wi, segs, nbands, band, H);
+                const bool border = at_border(it);
+                for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jg) {
+                    const uint32_t s = jg % kWsSlots, u = jg / kWsSlots;
+                    if (u > 0)
+                        ok = mbar_wait_ws(smem_u32(&empty_bar[s]), (u - 1) & 1u, &s_abort, lim);
+                    if (!ok) break;
+                    const uint32_t bar = smem_u32(border ? &raw_bar[s] : &full_bar[s]);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                                 "r"((uint32_t)S::kRowBytes)
+                                 : "memory");
+                    // the input gradient reads zeros outside the image, the
+                    // forward the nearest row
+                    const int sr = DGRAD ? r : min(max(r, 0), H - 1);
+                    asm volatile(
+                        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::"
+                        "complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(
+                            smem_u32(ring + s * S::kSlotBytes)),
+                        "l"(&xmap), "r"(0), "r"(it.x0 - 1), "r"(sr), "r"(it.b), "r"(bar)
+                        : "memory");
+                    if (border) raw ^= 1u << s;
+                    last_raw = (last_raw & ~(1u << s)) | ((border ? 1u : 0u) << s);
                 }
-                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(
-                                 smem_u32(&full_bar[s]))
-                             : "memory");
+            }
+            // no copy may land after this CTA has left
+            const volatile int no_abort = 0;
+            for (uint32_t j = jg > kWsSlots ? jg - kWsSlots : 0; j < jg; ++j) {
+                const uint32_t s = j % kWsSlots;
+                const bool landed =
+                    last_raw >> s & 1u
+                        ? mbar_wait_ws(smem_u32(&raw_bar[s]), (raw >> s & 1u) ^ 1u, &no_abort)
+                        : mbar_wait_ws(smem_u32(&full_bar[s]), (j / kWsSlots) & 1u, &no_abort);
+                ok = ok && landed;
             }
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp == 6) {
+        // ----------------------------------------------------------- borders
+        if constexpr (!DGRAD) {
+            constexpr int CPX = S::kPitch / 16;  // 16-byte chunks of a pixel
+            // chunk c of pixel p within a slot, as the swizzled copy places it
+            auto chunk_at = [](int p, int c) {
+                const int f = CPX == 8 ? p & 7 : CPX == 4 ? p >> 1 & 3 : p >> 2 & 1;
+                return p * S::kPitch + (c ^ f) * 16;
+            };
+            uint32_t jg = 0, raw = 0;
+            for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
+                const WsItem it = ws_item(wi, segs, nbands, band, H);
+                const int rows = it.y1 - it.y0 + 2;
+                if (!at_border(it)) {
+                    jg += rows;
+                    continue;
+                }
+                for (int i = 0; i < rows && ok; ++i, ++jg) {
+                    const uint32_t s = jg % kWsSlots;
+                    ok = __all_sync(0xffffffffu, mbar_wait_ws(smem_u32(&raw_bar[s]), raw >> s & 1u,
+                                                              &s_abort, lim));
+                    if (!ok) break;
+                    raw ^= 1u << s;
+                    uint8_t* slot = ring + s * S::kSlotBytes;
+                    const int last = W - it.x0;  // ring pixel of the image's last one
+                    if (lane < CPX && it.x0 == 0)
+                        *reinterpret_cast<uint4*>(slot + chunk_at(0, lane)) =
+                            *reinterpret_cast<const uint4*>(slot + chunk_at(1, lane));
+                    if (lane < CPX && last + 1 < kHaloPx)
+                        *reinterpret_cast<uint4*>(slot + chunk_at(last + 1, lane)) =
+                            *reinterpret_cast<const uint4*>(slot + chunk_at(last, lane));
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&full_bar[s]));
+                }
+            }
+        }
     } else if (warp == 4) {
         // --------------------------------------------------------------- MMA
-        if (lane == 0) {
-            const uint64_t a_hi = smem_desc(0, kHaloPx * 16, 128);
+        // every lane walks the rows (uniform control flow), one issues
+        {
+            // (the OR over the warp lands in a uniform register)
+            const uint32_t tmem_u = __reduce_or_sync(0xffffffffu, tmem);
+            const uint64_t a_hi = smem_desc_swizzled(0, S::kPitch);
             const uint64_t bd_base = smem_desc(smem_u32(sB), 3 * COUT * 16, 128);
             const uint32_t ring_a = smem_u32(ring);
             uint32_t jg = 0, og = 0;
@@ -645,23 +746,26 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
             for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
                 const WsItem it = ws_item(wi, segs, nbands, band, H);
                 for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jg) {
-                    ok = mbar_wait_ws(smem_u32(&full_bar[jg % kWsSlots]),
-                                      (jg / kWsSlots) & 1u, &s_abort, lim);
+                    ok = __all_sync(0xffffffffu,
+                                    mbar_wait_ws(smem_u32(&full_bar[jg % kWsSlots]),
+                                                 (jg / kWsSlots) & 1u, &s_abort, lim));
                     // dy blocks whose output row r + 1 - dy lies in [y0, y1)
                     const int dlo = max(0, r + 2 - it.y1), dhi = min(2, r + 1 - it.y0);
                     const int nd = dhi - dlo + 1;
                     const uint32_t o_first = og + (uint32_t)(r + 1 - dlo - it.y0);
                     if (ok && dlo == 0 && o_first >= (uint32_t)kAccSlots)
-                        ok = mbar_wait_ws(smem_u32(&free_bar[o_first % kAccSlots]),
-                                          ((o_first / kAccSlots) - 1) & 1u, &s_abort, lim);
+                        ok = __all_sync(0xffffffffu,
+                                        mbar_wait_ws(smem_u32(&free_bar[o_first % kAccSlots]),
+                                                     ((o_first / kAccSlots) - 1) & 1u, &s_abort,
+                                                     lim));
                     if (!ok) break;
                     // plan: outputs o_first, o_first - 1, ... in at most two
                     // runs of adjacent TMEM column blocks (split at the wrap)
                     const int m = (int)(o_first % kAccSlots);
                     const int len0 = nd < m + 1 ? nd : m + 1;
                     const int len1 = nd - len0;
-                    const uint32_t d0 = tmem + (uint32_t)(COUT * (kAccSlots - 1 - m));
-                    const uint32_t d1 = tmem;  // the run after the wrap starts at slot 0
+                    const uint32_t d0 = tmem_u + (uint32_t)(COUT * (kAccSlots - 1 - m));
+                    const uint32_t d1 = tmem_u;  // the run after the wrap starts at slot 0
                     const uint32_t id0 = idesc_for_rows(len0, COUT);
                     const uint32_t id1 = idesc_for_rows(len1 > 0 ? len1 : 1, COUT);
                     // B row offsets (16-byte units) of the first dy block of each run
@@ -670,18 +774,23 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
                     const uint64_t ad_row =
                         a_hi | (uint64_t)((ring_a + (jg % kWsSlots) * S::kSlotBytes) >> 4);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    auto issue = [&](auto two) {
 #pragma unroll
-                    for (int dx = 0; dx < 3; ++dx) {
+                        for (int dx = 0; dx < 3; ++dx) {
 #pragma unroll
-                        for (int ks = 0; ks < NCH / 2; ++ks) {
-                            // A: input view shifted by dx pixels, channel chunk 2 ks;
-                            // B: weights of (dx, chunk 2 ks)
-                            const uint64_t ad = ad_row + (uint64_t)(2 * ks * kHaloPx + dx);
-                            const uint64_t boff = (uint64_t)((dx * NCH + 2 * ks) * 3 * COUT);
-                            mma_bf16(d0, ad, b0 + boff, id0, 1u);
-                            if (len1 > 0) mma_bf16(d1, ad, b1 + boff, id1, 1u);
+                            for (int ks = 0; ks < NCH / 2; ++ks) {
+                                // A: input view shifted by dx pixels, channels from 16 ks;
+                                // B: weights of (dx, chunk 2 ks)
+                                const uint64_t ad =
+                                    ad_row + (uint64_t)((dx * S::kPitch + 32 * ks) >> 4);
+                                const uint64_t boff = (uint64_t)((dx * NCH + 2 * ks) * 3 * COUT);
+                                mma_bf16_warp(d0, ad, b0 + boff, id0);
+                                if (two.value) mma_bf16_warp(d1, ad, b1 + boff, id1);
+                            }
                         }
-                    }
+                    };
+                    if (len1 == 0) issue(Flag<false>{});
+                    else issue(Flag<true>{});
                     if constexpr (DGRAD) {
                         // ghost output rows -1 and H of the zero-padded
                         // transpose, folded into rows 0 and H - 1 (the
@@ -695,25 +804,25 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
                             const int dsrc = f == 0 ? 2 : 0;  // block of output row -1 / H
                             const uint32_t sl =
                                 (og + (uint32_t)(o - it.y0)) % (uint32_t)kAccSlots;
-                            const uint32_t dd = tmem + (uint32_t)(COUT * (kAccSlots - 1 - (int)sl));
+                            const uint32_t dd = tmem_u + (uint32_t)(COUT * (kAccSlots - 1 - (int)sl));
                             const uint32_t idf = idesc_for_rows(1, COUT);
 #pragma unroll
                             for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
                                 for (int ks = 0; ks < NCH / 2; ++ks) {
-                                    const uint64_t ad = ad_row + (uint64_t)(2 * ks * kHaloPx + dx);
+                                    const uint64_t ad = ad_row + (uint64_t)((dx * S::kPitch + 32 * ks) >> 4);
                                     const uint64_t boff =
                                         (uint64_t)((dx * NCH + 2 * ks) * 3 * COUT + dsrc * COUT);
-                                    mma_bf16(dd, ad, bd_base + boff, idf, 1u);
+                                    mma_bf16_warp(dd, ad, bd_base + boff, idf);
                                 }
                         }
                     }
-                    mma_commit(smem_u32(&empty_bar[jg % kWsSlots]));
+                    mma_commit_warp(smem_u32(&empty_bar[jg % kWsSlots]));
                     last_row = (int)jg;
                     if (dhi == 2) {
                         // output row r - 1 has all three contributions
                         const uint32_t o_done = og + (uint32_t)(r - 1 - it.y0);
-                        mma_commit(smem_u32(&outf_bar[o_done % kAccSlots]));
+                        mma_commit_warp(smem_u32(&outf_bar[o_done % kAccSlots]));
                         last_out = (int)o_done;
                     }
                 }
@@ -847,6 +956,35 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
     }
 }
 
+// The copy of one halo row: box of all channels x kHaloPx pixels of one row of
+// one image of x [B][H][W][cin], swizzled by the pixel's width.
+hp_status row_map(const void* x, int cin, int W, int H, int B, CUtensorMap* map)
+{
+    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+    if (!encode) {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
+                                                         cudaEnableDefault, &found);
+        if (e == cudaSuccess && found != cudaDriverEntryPointSuccess) e = cudaErrorNotSupported;
+        if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
+        encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+    }
+    const cuuint64_t pix = 2ull * cin;
+    const cuuint64_t dims[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+    const cuuint64_t strides[3] = {pix, pix * W, pix * W * H};
+    const cuuint32_t box[4] = {(cuuint32_t)cin, (cuuint32_t)kHaloPx, 1, 1};
+    const cuuint32_t one[4] = {1, 1, 1, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims,
+                              strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                              cin == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                              : cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                          : CU_TENSOR_MAP_SWIZZLE_32B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? HP_OK : HP_ERR_INVALID_ARG;
+}
+
 // warp-specialised row walk, one persistent CTA per SM; bands sized for about
 // eight work items per CTA (an image narrower than 128 pixels is one strip
 // whose pixels past its width are clamped on load and not stored)
@@ -856,6 +994,9 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
                     const void* act = nullptr, uint32_t wait_limit = 0, bool pdl = false)
 {
     using R = WsSmem<CIN, COUT, OUT1>;
+    CUtensorMap xmap;
+    hp_status mrc = row_map(x, CIN, W, H, B, &xmap);
+    if (mrc != HP_OK) return mrc;
     static bool rattr = false;
     if (!rattr) {
         cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_ws_kernel<CIN, COUT, OUT1, DGRAD>,
@@ -885,9 +1026,8 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, conv3x3_tc_ws_kernel<CIN, COUT, OUT1, DGRAD>,
-                                       (const uint4*)x, (const uint4*)w, bias, y, H, W, segs,
-                                       nbands, band, (int)items, relu, err, wait_limit,
-                                       (const uint4*)act);
+                                       (const uint4*)w, bias, y, H, W, segs, nbands, band,
+                                       (int)items, relu, err, wait_limit, (const uint4*)act, xmap);
     if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
     return check_launch();
 }
