@@ -426,6 +426,33 @@ __device__ __forceinline__ bool mbar_wait_ws(uint32_t mbar, uint32_t parity,
     return false;
 }
 
+// The same for four barriers and all lanes of a warp, looked at together.
+__device__ __forceinline__ bool mbar_wait4(const uint32_t (&mbar)[4], const uint32_t (&parity)[4],
+                                           const volatile int* abort_flag, uint32_t limit)
+{
+    bool ok = true;
+    if (limit == kWsSpinLimit) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred a, b, c, d;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 a, [%1], %2;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 b, [%3], %4;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 c, [%5], %6;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 d, [%7], %8;\n\t"
+            "and.pred a, a, b;\n\tand.pred c, c, d;\n\tand.pred a, a, c;\n\t"
+            "selp.u32 %0, 1, 0, a;\n\t}"
+            : "=r"(done)
+            : "r"(mbar[0]), "r"(parity[0]), "r"(mbar[1]), "r"(parity[1]), "r"(mbar[2]),
+              "r"(parity[2]), "r"(mbar[3]), "r"(parity[3])
+            : "memory");
+        if (__all_sync(0xffffffffu, done != 0)) return true;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        ok = ok && __all_sync(0xffffffffu, mbar_wait_ws(mbar[i], parity[i], abort_flag, limit));
+    return ok;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
@@ -560,11 +587,11 @@ __device__ __forceinline__ uint32_t idesc_for_rows(int n_out, int cout)
 // derivative of the layer that produced act; act may be null).
 template <int CIN, int COUT, bool OUT1, bool DGRAD = false>
 __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()))
-    conv3x3_tc_ws_kernel(const uint4* __restrict__ w,
-                         const float* __restrict__ bias, void* __restrict__ yout, int H, int W,
+    conv3x3_tc_ws_kernel(const float* __restrict__ bias, void* __restrict__ yout, int H, int W,
                          int segs, int nbands, int band, int items, int relu, int* err,
                          uint32_t wait_limit, const uint4* __restrict__ act,
-                         const __grid_constant__ CUtensorMap xmap)
+                         const __grid_constant__ CUtensorMap xmap,
+                         const __grid_constant__ CUtensorMap wmap)
 {
     using S = WsSmem<CIN, COUT, OUT1>;
     // polls of each pipeline wait before it gives up (0: the compiled limit);
@@ -576,6 +603,7 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
     uint8_t* ring = smem;
     uint8_t* sB = smem + S::kRingBytes;
     __shared__ __align__(8) uint64_t full_bar[kWsSlots];
+    __shared__ __align__(8) uint64_t w_bar;              // the weights are there
     __shared__ __align__(8) uint64_t raw_bar[kWsSlots];  // copied, borders not replicated yet
     __shared__ __align__(8) uint64_t empty_bar[kWsSlots];
     __shared__ __align__(8) uint64_t outf_bar[kAccSlots];
@@ -610,18 +638,23 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
                          "r"(4u));
         }
         s_abort = 0;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&w_bar)), "r"(1u));
         asm volatile("fence.mbarrier_init.release.cluster;");
+        // weights [tap = 3 dy + dx][cout][cin] -> [dx][dy][cout][cin], each
+        // tap one swizzled copy: for one dx the three dy blocks are adjacent
+        // along N.  They do not depend on the kernel before this one.
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&w_bar)),
+                     "r"((uint32_t)S::kBBytes)
+                     : "memory");
+        for (int tap = 0; tap < 9; ++tap)
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+                "[%0], [%1, {%2, %3}], [%4];" ::"r"(
+                    smem_u32(sB) + (uint32_t)((tap % 3 * 3 + tap / 3) * COUT * S::kPitch)),
+                "l"(&wmap), "r"(0), "r"(tap * COUT), "r"(smem_u32(&w_bar))
+                : "memory");
     }
     for (int i = tid; i < COUT; i += kWsThreads) s_bias[i] = bias[i];
-    // weights [tap = 3 dy + dx][cout][chunk] -> [dx][chunk][dy][cout] (16 B each)
-    for (int i = tid; i < 9 * COUT * NCH; i += kWsThreads) {
-        const int ch = i % NCH;
-        const int n = (i / NCH) % COUT;
-        const int tap = i / (NCH * COUT);
-        const int dy = tap / 3, dx = tap - 3 * (tap / 3);
-        const uint4 v = w[(size_t)(tap * COUT + n) * NCH + ch];
-        *reinterpret_cast<uint4*>(sB + (((dx * NCH + ch) * 3 + dy) * COUT + n) * 16) = v;
-    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -739,25 +772,38 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
             // (the OR over the warp lands in a uniform register)
             const uint32_t tmem_u = __reduce_or_sync(0xffffffffu, tmem);
             const uint64_t a_hi = smem_desc_swizzled(0, S::kPitch);
-            const uint64_t bd_base = smem_desc(smem_u32(sB), 3 * COUT * 16, 128);
+            const uint64_t bd_base = smem_desc_swizzled(smem_u32(sB), S::kPitch);
+            constexpr uint64_t kBlock = COUT * S::kPitch / 16;  // one dy block, 16-byte units
+            const volatile int never = 0;
+            ok = __all_sync(0xffffffffu, mbar_wait_ws(smem_u32(&w_bar), 0u, &never));
             const uint32_t ring_a = smem_u32(ring);
             uint32_t jg = 0, og = 0;
             int last_row = -1, last_out = -1;
             for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
                 const WsItem it = ws_item(wi, segs, nbands, band, H);
                 for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jg) {
-                    ok = __all_sync(0xffffffffu,
-                                    mbar_wait_ws(smem_u32(&full_bar[jg % kWsSlots]),
-                                                 (jg / kWsSlots) & 1u, &s_abort, lim));
                     // dy blocks whose output row r + 1 - dy lies in [y0, y1)
                     const int dlo = max(0, r + 2 - it.y1), dhi = min(2, r + 1 - it.y0);
                     const int nd = dhi - dlo + 1;
                     const uint32_t o_first = og + (uint32_t)(r + 1 - dlo - it.y0);
-                    if (ok && dlo == 0 && o_first >= (uint32_t)kAccSlots)
-                        ok = __all_sync(0xffffffffu,
-                                        mbar_wait_ws(smem_u32(&free_bar[o_first % kAccSlots]),
-                                                     ((o_first / kAccSlots) - 1) & 1u, &s_abort,
-                                                     lim));
+                    // the barriers of two rows are looked at together: a look
+                    // costs about 180 cycles (of 1,152 that a row's MMAs take)
+                    if (((r - it.y0) & 1) != 0) {
+                        const int n = r < it.y1 ? 2 : 1;  // rows r, r + 1
+                        uint32_t bar[4], par[4];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const uint32_t j = jg + (i < n ? i : 0);
+                            bar[2 * i] = smem_u32(&full_bar[j % kWsSlots]);
+                            par[2 * i] = (j / kWsSlots) & 1u;
+                            // output row r + 1 + i starts with this row, if the band has it
+                            const uint32_t o = og + (uint32_t)(r + 1 + i - it.y0);
+                            const bool starts = r + 1 + i < it.y1 && o >= (uint32_t)kAccSlots;
+                            bar[2 * i + 1] = starts ? smem_u32(&free_bar[o % kAccSlots]) : bar[0];
+                            par[2 * i + 1] = starts ? ((o / kAccSlots) - 1) & 1u : par[0];
+                        }
+                        ok = mbar_wait4(bar, par, &s_abort, lim);
+                    }
                     if (!ok) break;
                     // plan: outputs o_first, o_first - 1, ... in at most two
                     // runs of adjacent TMEM column blocks (split at the wrap)
@@ -768,9 +814,9 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
                     const uint32_t d1 = tmem_u;  // the run after the wrap starts at slot 0
                     const uint32_t id0 = idesc_for_rows(len0, COUT);
                     const uint32_t id1 = idesc_for_rows(len1 > 0 ? len1 : 1, COUT);
-                    // B row offsets (16-byte units) of the first dy block of each run
-                    const uint64_t b0 = bd_base + (uint64_t)(dlo * COUT);
-                    const uint64_t b1 = bd_base + (uint64_t)((dlo + len0) * COUT);
+                    // B: the first dy block of each run
+                    const uint64_t b0 = bd_base + (uint64_t)dlo * kBlock;
+                    const uint64_t b1 = bd_base + (uint64_t)(dlo + len0) * kBlock;
                     const uint64_t ad_row =
                         a_hi | (uint64_t)((ring_a + (jg % kWsSlots) * S::kSlotBytes) >> 4);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -780,10 +826,10 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
 #pragma unroll
                             for (int ks = 0; ks < NCH / 2; ++ks) {
                                 // A: input view shifted by dx pixels, channels from 16 ks;
-                                // B: weights of (dx, chunk 2 ks)
+                                // B: weights of dx, channels from 16 ks
                                 const uint64_t ad =
                                     ad_row + (uint64_t)((dx * S::kPitch + 32 * ks) >> 4);
-                                const uint64_t boff = (uint64_t)((dx * NCH + 2 * ks) * 3 * COUT);
+                                const uint64_t boff = 3 * dx * kBlock + 2 * ks;
                                 mma_bf16_warp(d0, ad, b0 + boff, id0);
                                 if (two.value) mma_bf16_warp(d1, ad, b1 + boff, id1);
                             }
@@ -811,8 +857,7 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
 #pragma unroll
                                 for (int ks = 0; ks < NCH / 2; ++ks) {
                                     const uint64_t ad = ad_row + (uint64_t)((dx * S::kPitch + 32 * ks) >> 4);
-                                    const uint64_t boff =
-                                        (uint64_t)((dx * NCH + 2 * ks) * 3 * COUT + dsrc * COUT);
+                                    const uint64_t boff = (3 * dx + dsrc) * kBlock + 2 * ks;
                                     mma_bf16_warp(dd, ad, bd_base + boff, idf);
                                 }
                         }
@@ -956,9 +1001,8 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
     }
 }
 
-// The copy of one halo row: box of all channels x kHaloPx pixels of one row of
-// one image of x [B][H][W][cin], swizzled by the pixel's width.
-hp_status row_map(const void* x, int cin, int W, int H, int B, CUtensorMap* map)
+// cuTensorMapEncodeTiled, by way of the runtime (no link to the driver library)
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 {
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     if (!encode) {
@@ -967,22 +1011,49 @@ hp_status row_map(const void* x, int cin, int W, int H, int B, CUtensorMap* map)
         cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
                                                          cudaEnableDefault, &found);
         if (e == cudaSuccess && found != cudaDriverEntryPointSuccess) e = cudaErrorNotSupported;
-        if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
-        encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+        if (e != cudaSuccess) set_cuda_error(e);
+        else encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     }
+    return encode;
+}
+
+// A map of BF16 data whose inner dimension is the channels of one pixel or
+// filter, swizzled by their width.
+hp_status channel_map(const void* p, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                      const cuuint32_t* box, CUtensorMap* map)
+{
+    const auto encode = tensor_map_encoder();
+    if (!encode) return HP_ERR_CUDA;
+    const cuuint32_t one[4] = {1, 1, 1, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank,
+                              const_cast<void*>(p), dims, strides, box, one,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE,
+                              dims[0] == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                              : dims[0] == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                              : CU_TENSOR_MAP_SWIZZLE_32B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? HP_OK : HP_ERR_INVALID_ARG;
+}
+
+// The copy of one halo row: all channels x kHaloPx pixels of one row of one
+// image of x [B][H][W][cin].
+hp_status row_map(const void* x, int cin, int W, int H, int B, CUtensorMap* map)
+{
     const cuuint64_t pix = 2ull * cin;
     const cuuint64_t dims[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
     const cuuint64_t strides[3] = {pix, pix * W, pix * W * H};
     const cuuint32_t box[4] = {(cuuint32_t)cin, (cuuint32_t)kHaloPx, 1, 1};
-    const cuuint32_t one[4] = {1, 1, 1, 1};
-    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims,
-                              strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              cin == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
-                              : cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                          : CU_TENSOR_MAP_SWIZZLE_32B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HP_OK : HP_ERR_INVALID_ARG;
+    return channel_map(x, 4, dims, strides, box, map);
+}
+
+// The copy of one tap of the weights [9][cout][cin].
+hp_status weight_map(const void* w, int cin, int cout, CUtensorMap* map)
+{
+    const cuuint64_t dims[2] = {(cuuint64_t)cin, 9ull * cout};
+    const cuuint64_t strides[1] = {2ull * cin};
+    const cuuint32_t box[2] = {(cuuint32_t)cin, (cuuint32_t)cout};
+    return channel_map(w, 2, dims, strides, box, map);
 }
 
 // warp-specialised row walk, one persistent CTA per SM; bands sized for about
@@ -994,8 +1065,9 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
                     const void* act = nullptr, uint32_t wait_limit = 0, bool pdl = false)
 {
     using R = WsSmem<CIN, COUT, OUT1>;
-    CUtensorMap xmap;
+    CUtensorMap xmap, wmap;
     hp_status mrc = row_map(x, CIN, W, H, B, &xmap);
+    if (mrc == HP_OK) mrc = weight_map(w, CIN, COUT, &wmap);
     if (mrc != HP_OK) return mrc;
     static bool rattr = false;
     if (!rattr) {
@@ -1026,8 +1098,8 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, conv3x3_tc_ws_kernel<CIN, COUT, OUT1, DGRAD>,
-                                       (const uint4*)w, bias, y, H, W, segs, nbands, band,
-                                       (int)items, relu, err, wait_limit, (const uint4*)act, xmap);
+                                       bias, y, H, W, segs, nbands, band, (int)items, relu, err,
+                                       wait_limit, (const uint4*)act, xmap, wmap);
     if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
     return check_launch();
 }
