@@ -289,12 +289,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     }
 }
 
-// Row-walking layout for width >= 128: a CTA walks a 128-pixel column strip
-// down a band of rows.  Input rows live once in a ring in shared memory,
-// [slot][chunk][130 pixels][8 channels] (pixels x0-1 .. x0+128, replicated at
-// the borders), so the A operand of tap (dy, dx) is a descriptor view of the
-// slot holding row y + dy - 1, shifted by dx pixels (16 bytes): LBO = 130 * 16
-// bytes between channel chunks, SBO = 128 bytes between groups of 8 pixels.
+// Row-walking layout: a CTA walks a 128-pixel column strip down its rows.
+// Input rows live once in a ring in shared memory, [slot][130 pixels][channels]
+// (pixels x0 - 1 .. x0 + 128, replicated at the borders), each one TMA copy
+// swizzled by the channels' width, so the A operand of tap (dy, dx) is a
+// descriptor view of the slot holding row y + dy - 1 that starts dx pixels on.
 constexpr int kHaloPx = kTileM + 2;
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
@@ -309,35 +308,35 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, 
                  "r"(valid ? 16u : 0u));
 }
 
-// Warp-specialised persistent row walk (width >= 128).  Each CTA loops over
-// work items (grid, 128-pixel column strip, band of rows); the input rows of
-// all its items form one stream through a kWsSlots-deep ring of halo rows in
-// shared memory (the layout and descriptor views above).
+// Warp-specialised persistent row walk.  Each CTA loops over items (grid,
+// 128-pixel column strip, rows of it); the input rows of all its items form
+// one stream through a kWsSlots-deep ring of halo rows in shared memory (the
+// layout and descriptor views above).
 //
 // One input row r feeds three output rows: r + 1 through the kernel row
 // dy = 0, r through dy = 1 and r - 1 through dy = 2.  The weights are staged
-// as [dx][chunk][dy][cout][8 channels], so for each (dx, K step) the three
+// as [dx][dy][cout][cin], so for each (dx, K step) the three
 // dy blocks are adjacent along N, and the accumulators of consecutive output
 // rows sit in adjacent TMEM column blocks of a ring of kAccSlots (output o of
 // the CTA's stream at columns Cout * (kAccSlots - 1 - o % kAccSlots)).  One
 // MMA with N = 3 Cout then adds row r's contribution to all three outputs:
 // the A operand (the 4 KB input view) is read once for three output rows,
-// and each input row needs 3 x Cin/16 MMAs.  At the first and last rows of a
-// band only the dy blocks whose output lies in the band are issued, and an
+// and each input row needs 3 x Cin/16 MMAs.  At the first and last rows of an
+// item only the dy blocks whose output lies in it are issued, and an
 // MMA whose column range would wrap around the ring is split in two; this
 // plan is made once per input row, so the unrolled issue loop costs two
 // descriptor additions per MMA.  Accumulator slots are pre-filled with the
 // bias, so every MMA accumulates.
 //
 // Roles, overlapping through mbarriers:
-//   warp 5 (producer): cp.async of input row j into slot j % kWsSlots once the
+//   warp 5 (producer): the copy of input row j into slot j % kWsSlots once the
 //     MMAs that read the slot's previous row have completed (empty[slot],
-//     arrived by tcgen05.commit); completion signalled with
-//     cp.async.mbarrier.arrive on full[slot];
-//   warp 4, one thread (MMA): per input row waits for the row and, when it
-//     starts a new output row, for that accumulator slot to be refilled;
-//     issues the MMAs, commits to empty[] of the row and, when an output row
-//     is complete, to out_full[] of its slot;
+//     arrived by tcgen05.commit);
+//   warp 6 (borders): replicates the border pixel of rows that need it;
+//   warp 4 (MMA, all lanes in step, one issues): per input row waits for the
+//     row and, when it starts a new output row, for that accumulator slot to
+//     be refilled; issues the MMAs, commits to empty[] of the row and, when an
+//     output row is complete, to out_full[] of its slot;
 //   warps 0-3 (epilogue): wait out_full, tcgen05.ld their 32 TMEM lanes,
 //     refill the slot with the bias (tcgen05.st) and release it (slot_free),
 //     then ReLU + BF16 rounding in one conversion and a store staged through
@@ -572,6 +571,33 @@ __device__ __forceinline__ WsItem ws_item(int w, int segs, int nbands, int band,
     return it;
 }
 
+// The rows of all strips (grid, 128-pixel column) form one sequence of `rows`
+// rows, and CTA k of n takes the k-th of n equal pieces of it, so that no CTA
+// has more than one row above the mean; an item is what of a piece lies in one
+// strip.  (Bands of a common height left 8 x 512^2 with 1,184 items for 152
+// CTAs, 8 x 14 rows with a halo of two each, where the mean is 107.8 rows.)
+struct WsRows {
+    int at, end;
+};
+
+__device__ __forceinline__ WsRows ws_rows(int rows)
+{
+    return {(int)((long long)rows * blockIdx.x / gridDim.x),
+            (int)((long long)rows * (blockIdx.x + 1) / gridDim.x)};
+}
+
+__device__ __forceinline__ WsItem ws_next(WsRows& piece, int segs, int H)
+{
+    WsItem it;
+    const int strip = piece.at / H;
+    it.b = strip / segs;
+    it.x0 = (strip - it.b * segs) * kTileM;
+    it.y0 = piece.at - strip * H;
+    it.y1 = min(H, it.y0 + piece.end - piece.at);
+    piece.at += it.y1 - it.y0;
+    return it;
+}
+
 __device__ __forceinline__ uint32_t idesc_for_rows(int n_out, int cout)
 {
     return n_out == 1 ? mma_idesc(kTileM, cout)
@@ -588,7 +614,7 @@ __device__ __forceinline__ uint32_t idesc_for_rows(int n_out, int cout)
 template <int CIN, int COUT, bool OUT1, bool DGRAD = false>
 __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()))
     conv3x3_tc_ws_kernel(const float* __restrict__ bias, void* __restrict__ yout, int H, int W,
-                         int segs, int nbands, int band, int items, int relu, int* err,
+                         int segs, int rows, int relu, int* err,
                          uint32_t wait_limit, const uint4* __restrict__ act,
                          const __grid_constant__ CUtensorMap xmap,
                          const __grid_constant__ CUtensorMap wmap)
@@ -692,8 +718,8 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
         if (lane == 0) {
             uint32_t jg = 0, raw = 0;  // raw: parity of the next phase of raw_bar[s]
             uint32_t last_raw = 0;     // bit s: the last copy into slot s signalled raw_bar
-            for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-                const WsItem it = ws_item(wi, segs, nbands, band, H);
+            for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+                const WsItem it = ws_next(piece, segs, H);
                 const bool border = at_border(it);
                 for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jg) {
                     const uint32_t s = jg % kWsSlots, u = jg / kWsSlots;
@@ -738,14 +764,14 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
                 return p * S::kPitch + (c ^ f) * 16;
             };
             uint32_t jg = 0, raw = 0;
-            for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-                const WsItem it = ws_item(wi, segs, nbands, band, H);
-                const int rows = it.y1 - it.y0 + 2;
+            for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+                const WsItem it = ws_next(piece, segs, H);
+                const int halo_rows = it.y1 - it.y0 + 2;
                 if (!at_border(it)) {
-                    jg += rows;
+                    jg += halo_rows;
                     continue;
                 }
-                for (int i = 0; i < rows && ok; ++i, ++jg) {
+                for (int i = 0; i < halo_rows && ok; ++i, ++jg) {
                     const uint32_t s = jg % kWsSlots;
                     ok = __all_sync(0xffffffffu, mbar_wait_ws(smem_u32(&raw_bar[s]), raw >> s & 1u,
                                                               &s_abort, lim));
@@ -779,8 +805,8 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
             const uint32_t ring_a = smem_u32(ring);
             uint32_t jg = 0, og = 0;
             int last_row = -1, last_out = -1;
-            for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-                const WsItem it = ws_item(wi, segs, nbands, band, H);
+            for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+                const WsItem it = ws_next(piece, segs, H);
                 for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jg) {
                     // dy blocks whose output row r + 1 - dy lies in [y0, y1)
                     const int dlo = max(0, r + 2 - it.y1), dhi = min(2, r + 1 - it.y0);
@@ -893,8 +919,8 @@ __global__ void __launch_bounds__(kWsThreads, (ws_ctas_per_sm<CIN, COUT, OUT1>()
         uint8_t* stage = sB + S::kBBytes + warp * 32 * COUT * 2;
         const bool do_relu = relu != 0;
         uint32_t og = 0;
-        for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-            const WsItem it = ws_item(wi, segs, nbands, band, H);
+        for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+            const WsItem it = ws_next(piece, segs, H);
             for (int yy = it.y0; yy < it.y1; ++yy, ++og) {
                 const uint32_t sl = og % kAccSlots;
                 // DGRAD: this lane's activation chunks of the row, loaded while
@@ -1056,9 +1082,8 @@ hp_status weight_map(const void* w, int cin, int cout, CUtensorMap* map)
     return channel_map(w, 2, dims, strides, box, map);
 }
 
-// warp-specialised row walk, one persistent CTA per SM; bands sized for about
-// eight work items per CTA (an image narrower than 128 pixels is one strip
-// whose pixels past its width are clamped on load and not stored)
+// warp-specialised row walk, kCtas persistent CTAs per SM (an image narrower
+// than 128 pixels is one strip whose pixels past its width are not stored)
 template <int CIN, int COUT, bool OUT1, bool DGRAD = false>
 hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, int B, int H,
                     int W, int relu, int* err, int nsm, cudaStream_t st,
@@ -1080,12 +1105,8 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
     const int segs = (W + kTileM - 1) / kTileM;
     const long rows = (long)B * H * segs;
     const long ctas = (long)R::kCtas * nsm;
-    int band = (int)((rows + 8L * ctas - 1) / (8L * ctas));
-    band = band < 4 ? 4 : band > H ? H : band;
-    const int nbands = (H + band - 1) / band;
-    const long items = (long)B * segs * nbands;
-    if (items > 0x7fffffffL) return HP_ERR_INVALID_ARG;
-    const int grid = items < ctas ? (int)items : (int)ctas;
+    if (rows > 0x7fffffffL) return HP_ERR_INVALID_ARG;
+    const int grid = rows < ctas ? (int)rows : (int)ctas;
     // pdl: a programmatic dependent of the kernel before it in the stream
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -1098,7 +1119,7 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, conv3x3_tc_ws_kernel<CIN, COUT, OUT1, DGRAD>,
-                                       bias, y, H, W, segs, nbands, band, (int)items, relu, err,
+                                       bias, y, H, W, segs, (int)rows, relu, err,
                                        wait_limit, (const uint4*)act, xmap, wmap);
     if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
     return check_launch();
