@@ -296,18 +296,6 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 // descriptor view of the slot holding row y + dy - 1 that starts dx pixels on.
 constexpr int kHaloPx = kTileM + 2;
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src));
-}
-
-// 16 bytes from global memory, or 16 zero bytes when !valid (src is not read)
-__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, bool valid)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-                 "r"(valid ? 16u : 0u));
-}
-
 // Warp-specialised persistent row walk.  Each CTA loops over items (grid,
 // 128-pixel column strip, rows of it); the input rows of all its items form
 // one stream through a kWsSlots-deep ring of halo rows in shared memory (the
@@ -457,13 +445,6 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mbar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t mbar)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-        : "memory");
-}
-
 // 32 consecutive 32-bit TMEM columns of this thread's lane, without the wait.
 __device__ __forceinline__ void tmem_ld32_raw(uint32_t taddr, uint32_t* r)
 {
@@ -557,19 +538,6 @@ struct Flag {
 struct WsItem {
     int b, x0, y0, y1;
 };
-
-__device__ __forceinline__ WsItem ws_item(int w, int segs, int nbands, int band, int H)
-{
-    WsItem it;
-    const int seg = w % segs;
-    const int t = w / segs;
-    const int bi = t % nbands;
-    it.b = t / nbands;
-    it.x0 = seg * kTileM;
-    it.y0 = bi * band;
-    it.y1 = min(H, it.y0 + band);
-    return it;
-}
 
 // The rows of all strips (grid, 128-pixel column) form one sequence of `rows`
 // rows, and CTA k of n takes the k-th of n equal pieces of it, so that no CTA
@@ -1062,14 +1030,14 @@ hp_status channel_map(const void* p, int rank, const cuuint64_t* dims, const cuu
     return r == CUDA_SUCCESS ? HP_OK : HP_ERR_INVALID_ARG;
 }
 
-// The copy of one halo row: all channels x kHaloPx pixels of one row of one
-// image of x [B][H][W][cin].
-hp_status row_map(const void* x, int cin, int W, int H, int B, CUtensorMap* map)
+// The copy of one row: all channels x px pixels of one row of one image of
+// x [B][H][W][cin].
+hp_status row_map(const void* x, int cin, int W, int H, int B, int px, CUtensorMap* map)
 {
     const cuuint64_t pix = 2ull * cin;
     const cuuint64_t dims[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
     const cuuint64_t strides[3] = {pix, pix * W, pix * W * H};
-    const cuuint32_t box[4] = {(cuuint32_t)cin, (cuuint32_t)kHaloPx, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)cin, (cuuint32_t)px, 1, 1};
     return channel_map(x, 4, dims, strides, box, map);
 }
 
@@ -1091,7 +1059,7 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
 {
     using R = WsSmem<CIN, COUT, OUT1>;
     CUtensorMap xmap, wmap;
-    hp_status mrc = row_map(x, CIN, W, H, B, &xmap);
+    hp_status mrc = row_map(x, CIN, W, H, B, kHaloPx, &xmap);
     if (mrc == HP_OK) mrc = weight_map(w, CIN, COUT, &wmap);
     if (mrc != HP_OK) return mrc;
     static bool rattr = false;
@@ -1129,66 +1097,81 @@ hp_status launch_ws(const void* x, const void* w, const float* bias, void* y, in
 // Weight gradient of a 3 x 3 convolution with replicated borders on the
 // tensor cores:
 //     gW[dy][dx][co][ci] = sum over pixels p of gy[p][co] * x[clamp(p + (dy, dx))][ci]
-// Per 128-pixel row segment of an output-gradient row r this is a GEMM over
-// K = the 130 input pixels x0 - 1 .. x0 + 128 (padded to 144, 9 steps of 16):
-//   A = input rows (M = 128 = kRows rows x CI channels), taken MN-major straight
-//       from an input-row ring laid out [row][channel chunk][pixel][8 channels]
-//       with replicated halo pixels; consecutive rows are adjacent in shared
-//       memory (the first kRows - 1 ring slots are mirrored after the last),
-//       so one descriptor spans kRows rows;
-//   B = the gradient row in three copies shifted by dx (pixel q of copy dx
-//       holds gy[q - dx], zero outside the segment), N = 3 CO, MN-major;
-//   D = TMEM, lane (row i of the tile, ci), column (dx, co), accumulating over
-//       every row and segment the CTA visits.
-// CI = 64: two tiles per gradient row, input rows (r-1, r) and (r, r+1) (the
-// second tile's r half repeats the first and is not read out); CI = 32: one
-// tile of rows r-1 .. r+2 (the r+2 quarter is not read out and may hold any
-// row).  Warps 0-3 load (cp.async) and finally read the accumulators out to
-// per-CTA partial sums part[cta][3 dy + dx][co][ci]; warp 4 issues the MMAs.
-constexpr int kWgPx = 144;
-constexpr int kWgThreads = 160;
+// Per input row r and 128-pixel segment this is a GEMM over K = the segment's
+// output-gradient pixels (8 steps of 16, fewer at the image's right end):
+//   A = the input row, M = 128 = kShifts blocks of CI channels, block i the
+//       row shifted by i pixels: the rows are single TMA copies (130 pixels,
+//       the border pixels replicated by a helper warp), MN-major and swizzled
+//       by the channels' width, so a shift by one pixel is a stride of one
+//       pixel between the blocks;
+//   B = the gradient rows r - 1, r, r + 1 as far as the CTA has them, up to
+//       three consecutive slots of a ring of TMA copies, N = 3 CO;
+//   D = TMEM, lane (dx, ci), column (2 - dy, co), accumulating over every row
+//       and segment the CTA visits.
+// CI = 64: two tiles, dx 0 and 1, then dx 2 (the other half of the second is
+// not read out); CI = 32: one tile of dx 0..3 (3 is not read out).  Each
+// gradient pixel is a K index once, so no operand is staged in shifted copies.
+//
+// What bounds it: the MMAs, 2 x 8 x 96 cycles per row and segment at 64 -> 64
+// (N / 2 each), of which 3/4 are useful.  The gradient of a training batch of
+// 64 x 128^2 (13 of these layers) took 4.33 ms with three shifted copies of
+// the gradient row staged by cp.async, 18 MMAs per row issued from a branch of
+// one lane and bands of a common height, and takes 3.40 ms in this form.
+//
+// Roles: warp 5 copies the rows; warp 6 replicates the border pixels; warp 4
+// issues the MMAs, all lanes in step as in the forward; warps 0-3 add the
+// gradient rows up for the bias gradient while they are in shared memory, and
+// finally read the accumulators out to per-CTA partial sums
+// part[cta][3 dy + dx][co][ci].
+constexpr int kWgXSlots = 4;
+constexpr int kWgGSlots = 8;
+constexpr int kWgThreads = 224;
 
 template <int CI, int CO>
 struct WgSmem {
-    static constexpr int kChunksX = CI / 8, kChunksG = CO / 8;
-    // bytes per channel chunk of a row: 144 pixels plus 16 bytes, so that the
-    // chunks of one pixel fall in different shared-memory banks (the
-    // producers write them together)
-    static constexpr int kStride = kWgPx * 16 + 16;
-    static constexpr int kSlotBytes = kChunksX * kStride;
-    static constexpr int kRows = 128 / CI;
-    static constexpr int kSlots = kRows == 2 ? 4 : 5;
-    static constexpr int kMirror = kRows - 1;
-    static constexpr int kRingBytes = (kSlots + kMirror) * kSlotBytes;
-    static constexpr int kGBytes = 3 * kChunksG * kStride;
-    static constexpr int kTiles = kRows == 2 ? 2 : 1;
+    static constexpr int kPitchX = 2 * CI, kPitchG = 2 * CO;  // bytes of a pixel
+    static constexpr int kShifts = 128 / CI;
+    static constexpr int kTiles = kShifts == 2 ? 2 : 1;
+    static constexpr int kXRowBytes = kHaloPx * kPitchX, kGRowBytes = kTileM * kPitchG;
+    // the last tile's unread block reaches one pixel past the halo row
+    static constexpr int kXSlotBytes = ((kHaloPx + 1) * kPitchX + 1023) / 1024 * 1024;
+    static constexpr int kGOffset = kWgXSlots * kXSlotBytes;
+    static constexpr int kBytes = kGOffset + kWgGSlots * kGRowBytes;
     static constexpr int kN = 3 * CO;
-    static constexpr int kBytes = kRingBytes + 2 * kGBytes;
     static constexpr int kTmemCols = kTiles * kN <= 128 ? 128 : kTiles * kN <= 256 ? 256 : 512;
     static_assert(CI == 32 || CI == 64, "input channels 32 or 64");
     static_assert(CO == 32 || CO == 64, "output channels 32 or 64");
+    static_assert(kGRowBytes % 1024 == 0, "gradient slots on swizzle atoms");
     static_assert(kBytes <= 227 * 1024, "shared memory");
 };
 
+// Descriptor of an MN-major operand of pixels (K) by channels, swizzled by
+// the pixel pitch: `block` bytes between blocks of one pitch along M or N,
+// groups of eight pixels contiguous.
+__device__ __forceinline__ uint64_t smem_desc_pixels(uint32_t addr, int pitch, uint32_t block)
+{
+    return smem_desc(addr, block, 8 * pitch) | (pitch == 128 ? 2ull : 4ull) << 61;
+}
+
 template <int CI, int CO>
 __global__ void __launch_bounds__(kWgThreads, 1)
-    conv3x3_wgrad_tc_kernel(const uint4* __restrict__ x, const uint4* __restrict__ gy,
-                            float* __restrict__ part, float* __restrict__ partb, int H, int W,
-                            int segs, int nbands, int band, int items, int* err,
-                            uint32_t wait_limit)
+    conv3x3_wgrad_tc_kernel(float* __restrict__ part, float* __restrict__ partb, int H, int W,
+                            int segs, int rows, int* err, uint32_t wait_limit,
+                            const __grid_constant__ CUtensorMap xmap,
+                            const __grid_constant__ CUtensorMap gmap)
 {
     using S = WgSmem<CI, CO>;
     // polls of each pipeline wait before it gives up (0: the compiled limit);
-    // the waits for the issued MMAs (done_bar) always use the compiled limit
+    // the waits for issued MMAs and copies always use the compiled limit
     const uint32_t lim = wait_limit ? wait_limit : kWsSpinLimit;
-    constexpr int NX = S::kChunksX, NG = S::kChunksG;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* ring = smem;
-    uint8_t* gbuf = smem + S::kRingBytes;
-    __shared__ __align__(8) uint64_t xfull[S::kSlots];
-    __shared__ __align__(8) uint64_t xempty[S::kSlots];
-    __shared__ __align__(8) uint64_t gfull[2];
-    __shared__ __align__(8) uint64_t gempty[2];
+    uint8_t* xring = smem;
+    uint8_t* gring = smem + S::kGOffset;
+    __shared__ __align__(8) uint64_t xfull[kWgXSlots];
+    __shared__ __align__(8) uint64_t xraw[kWgXSlots];  // copied, borders not replicated yet
+    __shared__ __align__(8) uint64_t xempty[kWgXSlots];
+    __shared__ __align__(8) uint64_t gfull[kWgGSlots];
+    __shared__ __align__(8) uint64_t gempty[kWgGSlots];
     __shared__ __align__(8) uint64_t done_bar;
     __shared__ uint32_t tmem_base;
     __shared__ volatile int s_abort;
@@ -1197,9 +1180,6 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
-    // bias-gradient partial sums of the producer threads: channels 8 (tid % NG)
-    // .. + 7 over the pixels of every gradient row this CTA loads
-    float bacc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -1208,200 +1188,254 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int i = 0; i < S::kSlots; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&xfull[i])),
-                         "r"(128u));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&xempty[i])),
-                         "r"(1u));
+        auto init = [](uint64_t* bar, uint32_t count) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+        };
+        for (int i = 0; i < kWgXSlots; ++i) {
+            init(&xfull[i], 1);
+            init(&xraw[i], 1);
+            init(&xempty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&gfull[i])),
-                         "r"(128u));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&gempty[i])),
-                         "r"(1u));
+        for (int i = 0; i < kWgGSlots; ++i) {
+            init(&gfull[i], 1);
+            init(&gempty[i], 5);  // the MMAs and the four bias warps
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&done_bar)),
-                     "r"(1u));
+        init(&done_bar, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-    // pixels 130..143 of every input row are never loaded: zero them once so
-    // that the MMAs read finite values there (the gradient copies are zero
-    // at those pixels)
-    for (int i = tid; i < (S::kSlots + S::kMirror) * NX * (kWgPx - kHaloPx); i += kWgThreads) {
-        const int px = kHaloPx + i % (kWgPx - kHaloPx);
-        const int ch = (i / (kWgPx - kHaloPx)) % NX;
-        const int sl = i / ((kWgPx - kHaloPx) * NX);
-        *reinterpret_cast<uint4*>(ring + sl * S::kSlotBytes + ch * S::kStride + px * 16) =
-            make_uint4(0u, 0u, 0u, 0u);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
+    if (warp < 4) {  // every MMA accumulates
+        uint32_t zero[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) zero[i] = 0u;
+        for (int c = 0; c < S::kTiles * S::kN; c += 32)
+            tmem_st32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, zero);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     bool ok = true;
+    const volatile int no_abort = 0;
+    float bacc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 
-    if (warp < 4) {
+    auto at_border = [&](const WsItem& it) { return it.x0 == 0 || it.x0 + kHaloPx - 1 > W; };
+    if (warp == 5) {
         // ---------------------------------------------------------- producer
-        uint32_t xpos = 0, gcnt = 0;
-        uint4 pend[NG];
-#pragma unroll
-        for (int i = 0; i < NG; ++i) pend[i] = make_uint4(0u, 0u, 0u, 0u);
-        auto add_pend = [&]() {
-#pragma unroll
-            for (int i = 0; i < NG; ++i) {
-                const uint32_t e[4] = {pend[i].x, pend[i].y, pend[i].z, pend[i].w};
-#pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    bacc[2 * h] += __uint_as_float(e[h] << 16);
-                    bacc[2 * h + 1] += __uint_as_float(e[h] & 0xFFFF0000u);
+        if (lane == 0) {
+            uint32_t jx = 0, jg = 0, raw = 0;  // raw: parity of the next phase of xraw[s]
+            uint32_t last_raw = 0;  // bit s: the last copy into slot s signalled xraw
+            auto copy_row = [&](uint32_t dst, const CUtensorMap& map, uint32_t bytes, int x, int y,
+                                int b, uint32_t bar) {
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                             "r"(bytes)
+                             : "memory");
+                asm volatile(
+                    "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::"
+                    "complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+                    "l"(&map), "r"(0), "r"(x), "r"(y), "r"(b), "r"(bar)
+                    : "memory");
+            };
+            for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+                const WsItem it = ws_next(piece, segs, H);
+                const bool border = at_border(it);
+                for (int r = it.y0 - 1; r <= it.y1 && ok; ++r) {
+                    if (r + 1 < it.y1) {  // the gradient row that input row r is the first to need
+                        const uint32_t s = jg % kWgGSlots, u = jg / kWgGSlots;
+                        if (u > 0)
+                            ok = mbar_wait_ws(smem_u32(&gempty[s]), (u - 1) & 1u, &s_abort, lim);
+                        if (!ok) break;
+                        copy_row(smem_u32(gring + s * S::kGRowBytes), gmap, S::kGRowBytes, it.x0,
+                                 r + 1, it.b, smem_u32(&gfull[s]));
+                        ++jg;
+                    }
+                    const uint32_t s = jx % kWgXSlots, u = jx / kWgXSlots;
+                    if (u > 0)
+                        ok = mbar_wait_ws(smem_u32(&xempty[s]), (u - 1) & 1u, &s_abort, lim);
+                    if (!ok) break;
+                    copy_row(smem_u32(xring + s * S::kXSlotBytes), xmap, S::kXRowBytes, it.x0 - 1,
+                             min(max(r, 0), H - 1), it.b, smem_u32(border ? &xraw[s] : &xfull[s]));
+                    ++jx;
+                    if (border) raw ^= 1u << s;
+                    last_raw = (last_raw & ~(1u << s)) | ((border ? 1u : 0u) << s);
                 }
-                pend[i] = make_uint4(0u, 0u, 0u, 0u);
             }
+            if (!ok) s_abort = 1;
+            // no copy may land after this CTA has left
+            for (uint32_t j = jx > kWgXSlots ? jx - kWgXSlots : 0; j < jx; ++j) {
+                const uint32_t s = j % kWgXSlots;
+                const bool landed =
+                    last_raw >> s & 1u
+                        ? mbar_wait_ws(smem_u32(&xraw[s]), (raw >> s & 1u) ^ 1u, &no_abort)
+                        : mbar_wait_ws(smem_u32(&xfull[s]), (j / kWgXSlots) & 1u, &no_abort);
+                ok = ok && landed;
+            }
+            for (uint32_t j = jg > kWgGSlots ? jg - kWgGSlots : 0; j < jg; ++j)
+                ok = mbar_wait_ws(smem_u32(&gfull[j % kWgGSlots]), (j / kWgGSlots) & 1u, &no_abort) &&
+                     ok;
+        }
+    } else if (warp == 6) {
+        // ----------------------------------------------------------- borders
+        constexpr int CPX = S::kPitchX / 16;  // 16-byte chunks of a pixel
+        // chunk c of pixel p within a slot, as the swizzled copy places it
+        auto chunk_at = [](int p, int c) {
+            return p * S::kPitchX + (c ^ (CPX == 8 ? p & 7 : p >> 1 & 3)) * 16;
         };
-        auto load_x = [&](int b, int x0, int r, uint32_t pos) -> bool {
-            const uint32_t sl = pos % S::kSlots, u = pos / S::kSlots;
-            if (u > 0 && !mbar_wait_ws(smem_u32(&xempty[sl]), (u - 1) & 1u, &s_abort, lim))
-                return false;
-            const int sr = min(max(r, 0), H - 1);
-            const uint4* src_row = x + ((size_t)b * H + sr) * W * NX;
-            const uint32_t dst = smem_u32(ring + sl * S::kSlotBytes);
-            const uint32_t dst2 = smem_u32(ring + (S::kSlots + sl) * S::kSlotBytes);
-            for (int q = tid; q < kHaloPx * NX; q += 128) {
-                const int ch = q % NX, px = q / NX;
-                const int sx = min(max(x0 - 1 + px, 0), W - 1);
-                const uint4* src = src_row + (size_t)sx * NX + ch;
-                const uint32_t off = (uint32_t)(ch * S::kStride + px * 16);
-                cp_async16(dst + off, src);
-                if (sl < (uint32_t)S::kMirror) cp_async16(dst2 + off, src);
+        uint32_t jx = 0, raw = 0;
+        for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+            const WsItem it = ws_next(piece, segs, H);
+            const int halo_rows = it.y1 - it.y0 + 2;
+            if (!at_border(it)) {
+                jx += halo_rows;
+                continue;
             }
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(
-                             smem_u32(&xfull[sl]))
-                         : "memory");
-            return true;
-        };
-        auto load_g = [&](int b, int x0, int r, uint32_t cnt) -> bool {
-            const uint32_t bb = cnt & 1u, u = cnt >> 1;
-            if (u > 0 && !mbar_wait_ws(smem_u32(&gempty[bb]), (u - 1) & 1u, &s_abort, lim))
-                return false;
-            const uint4* src_row = gy + ((size_t)b * H + r) * W * NG;
-            const uint32_t dst = smem_u32(gbuf + bb * S::kGBytes);
-            const int xend = min(x0 + kTileM, W);
-            for (int q = tid; q < 3 * kWgPx * NG; q += 128) {
-                const int ch = q % NG, k = (q / NG) % kWgPx, dx = q / (NG * kWgPx);
-                const int col = x0 + k - dx;  // gradient pixel at input pixel x0 - 1 + k
-                const bool valid = col >= x0 && col < xend;
-                const uint4* src = src_row + (size_t)(valid ? col : x0) * NG + ch;
-                cp_async16_zfill(dst + (uint32_t)((dx * NG + ch) * S::kStride + k * 16), src, valid);
-            }
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(
-                             smem_u32(&gfull[bb]))
-                         : "memory");
-            // bias sums: the previous row's values (loaded one row earlier, so
-            // that their latency overlaps) are added, this row's are loaded
-            add_pend();
-            const int chb = tid % NG;
-#pragma unroll
-            for (int i = 0; i < NG; ++i) {
-                const int j = tid / NG + i * (128 / NG);
-                pend[i] = x0 + j < xend ? src_row[(size_t)(x0 + j) * NG + chb]
-                                        : make_uint4(0u, 0u, 0u, 0u);
-            }
-            return true;
-        };
-        for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-            const WsItem it = ws_item(wi, segs, nbands, band, H);
-            ok = load_x(it.b, it.x0, it.y0 - 1, xpos++) && load_x(it.b, it.x0, it.y0, xpos++);
-            for (int r = it.y0; r < it.y1 && ok; ++r) {
-                ok = load_x(it.b, it.x0, r + 1, xpos++) && load_g(it.b, it.x0, r, gcnt++);
+            for (int i = 0; i < halo_rows && ok; ++i, ++jx) {
+                const uint32_t s = jx % kWgXSlots;
+                ok = __all_sync(0xffffffffu,
+                                mbar_wait_ws(smem_u32(&xraw[s]), raw >> s & 1u, &s_abort, lim));
+                if (!ok) break;
+                raw ^= 1u << s;
+                uint8_t* slot = xring + s * S::kXSlotBytes;
+                const int last = W - it.x0;  // ring pixel of the image's last one
+                if (lane < CPX && it.x0 == 0)
+                    *reinterpret_cast<uint4*>(slot + chunk_at(0, lane)) =
+                        *reinterpret_cast<const uint4*>(slot + chunk_at(1, lane));
+                if (lane < CPX && last + 1 < kHaloPx)
+                    *reinterpret_cast<uint4*>(slot + chunk_at(last + 1, lane)) =
+                        *reinterpret_cast<const uint4*>(slot + chunk_at(last, lane));
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&xfull[s]));
             }
         }
-        add_pend();
-        if (!ok) s_abort = 1;  // the MMA thread stops waiting for rows
-        asm volatile("cp.async.wait_all;" ::: "memory");
-    } else if (lane == 0) {
+    } else if (warp == 4) {
         // --------------------------------------------------------------- MMA
-        constexpr uint32_t idesc = mma_idesc(128, S::kN) | (1u << 15) | (1u << 16);
-        const uint32_t ring_a = smem_u32(ring), g_a = smem_u32(gbuf);
-        uint32_t xpos = 0, gcnt = 0;
-        bool first = true;
-        for (int wi = blockIdx.x; wi < items && ok; wi += gridDim.x) {
-            const WsItem it = ws_item(wi, segs, nbands, band, H);
-            const uint32_t p0 = xpos;
-            const int nb = it.y1 - it.y0;
-            for (int i = 0; i < nb && ok; ++i) {
-                // input rows at positions p0 + i .. p0 + i + 2 (the first two
-                // were waited for by the previous row unless i == 0)
-                for (uint32_t pos = p0 + (i == 0 ? 0u : (uint32_t)i + 2u);
-                     pos <= p0 + (uint32_t)i + 2u && ok; ++pos)
-                    ok = mbar_wait_ws(smem_u32(&xfull[pos % S::kSlots]),
-                                      (pos / S::kSlots) & 1u, &s_abort, lim);
-                if (ok)
-                    ok = mbar_wait_ws(smem_u32(&gfull[gcnt & 1u]), (gcnt >> 1) & 1u, &s_abort,
-                                      lim);
+        constexpr uint32_t kMnMajor = (1u << 15) | (1u << 16);
+        const uint32_t tmem_u = __reduce_or_sync(0xffffffffu, tmem);
+        const uint64_t a_base = smem_desc_pixels(smem_u32(xring), S::kPitchX, S::kPitchX);
+        const uint64_t b_base = smem_desc_pixels(smem_u32(gring), S::kPitchG, S::kGRowBytes);
+        uint32_t jx = 0, jg = 0;  // jg: ring position of the item's first gradient row
+        for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+            const WsItem it = ws_next(piece, segs, H);
+            const int ksteps = (min(W - it.x0, kTileM) + 15) / 16;
+            for (int r = it.y0 - 1; r <= it.y1 && ok; ++r, ++jx) {
+                const uint32_t xs = jx % kWgXSlots;
+                // the row and the gradient row that it is the first to need
+                const bool more = r + 1 < it.y1;
+                const uint32_t gn = jg + (uint32_t)(r + 1 - it.y0);
+                uint32_t bar[4], par[4];
+                bar[0] = bar[2] = bar[3] = smem_u32(&xfull[xs]);
+                par[0] = par[2] = par[3] = (jx / kWgXSlots) & 1u;
+                bar[1] = more ? smem_u32(&gfull[gn % kWgGSlots]) : bar[0];
+                par[1] = more ? (gn / kWgGSlots) & 1u : par[0];
+                ok = mbar_wait4(bar, par, &s_abort, lim);
                 if (!ok) break;
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                // gradient rows g0 .. g0 + n - 1, at most two runs of
+                // adjacent slots (split where the ring wraps)
+                const int g0 = max(r - 1, it.y0), n = min(r + 1, it.y1 - 1) - g0 + 1;
+                const uint32_t s0 = (jg + (uint32_t)(g0 - it.y0)) % kWgGSlots;
+                const int len0 = min(n, kWgGSlots - (int)s0), len1 = n - len0;
+                const uint32_t d0 = tmem_u + (uint32_t)((g0 - r + 1) * CO);
+                const uint32_t d1 = d0 + (uint32_t)(len0 * CO);
+                const uint32_t id0 = idesc_for_rows(len0, CO) | kMnMajor;
+                const uint32_t id1 = idesc_for_rows(len1 > 0 ? len1 : 1, CO) | kMnMajor;
+                const uint64_t a = a_base + (uint64_t)(xs * S::kXSlotBytes >> 4);
+                const uint64_t b0 = b_base + (uint64_t)(s0 * S::kGRowBytes >> 4);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t gb_a = g_a + (gcnt & 1u) * S::kGBytes;
+                auto step = [&](int ks, auto two) {
 #pragma unroll
-                for (int t = 0; t < S::kTiles; ++t) {
-                    const uint32_t a0 = ring_a + ((p0 + (uint32_t)(i + t)) % S::kSlots) * S::kSlotBytes;
-#pragma unroll
-                    for (int ks = 0; ks < kWgPx / 16; ++ks) {
-                        const uint64_t ad = smem_desc(a0 + ks * 256, 128, S::kStride);
-                        const uint64_t bd = smem_desc(gb_a + ks * 256, 128, S::kStride);
-                        mma_bf16(tmem + (uint32_t)(t * S::kN), ad, bd, idesc,
-                                 (first && ks == 0) ? 0u : 1u);
+                    for (int t = 0; t < S::kTiles; ++t) {
+                        const uint64_t ad = a + (uint64_t)((16 * ks + 2 * t) * S::kPitchX >> 4);
+                        const uint64_t boff = (uint64_t)(16 * ks * S::kPitchG >> 4);
+                        mma_bf16_warp(d0 + (uint32_t)(t * S::kN), ad, b0 + boff, id0);
+                        if (two.value)  // continues at slot 0
+                            mma_bf16_warp(d1 + (uint32_t)(t * S::kN), ad, b_base + boff, id1);
                     }
-                }
-                first = false;
-                mma_commit(smem_u32(&gempty[gcnt & 1u]));
-                ++gcnt;
-                // input row p0 + i is not read again; after the last row of the
-                // item neither are the two after it
-                mma_commit(smem_u32(&xempty[(p0 + (uint32_t)i) % S::kSlots]));
-                if (i == nb - 1) {
-                    mma_commit(smem_u32(&xempty[(p0 + (uint32_t)i + 1u) % S::kSlots]));
-                    mma_commit(smem_u32(&xempty[(p0 + (uint32_t)i + 2u) % S::kSlots]));
+                };
+                auto issue = [&](auto two) {
+                    if (ksteps == kTileM / 16) {
+#pragma unroll
+                        for (int ks = 0; ks < kTileM / 16; ++ks) step(ks, two);
+                    } else {
+                        for (int ks = 0; ks < ksteps; ++ks) step(ks, two);
+                    }
+                };
+                if (len1 == 0) issue(Flag<false>{});
+                else issue(Flag<true>{});
+                mma_commit_warp(smem_u32(&xempty[xs]));
+                // gradient row r - 1 is not read again
+                if (r > it.y0) {
+                    const uint32_t gd = jg + (uint32_t)(r - 1 - it.y0);
+                    mma_commit_warp(smem_u32(&gempty[gd % kWgGSlots]));
                 }
             }
-            xpos = p0 + (uint32_t)nb + 2u;
+            jg += (uint32_t)(it.y1 - it.y0);
         }
         if (!ok) s_abort = 1;
         // every MMA issued must have landed before the accumulators are read
         // or freed, also on the error path
-        mma_commit(smem_u32(&done_bar));
-        const volatile int no_abort = 0;
-        if (!mbar_wait_ws(smem_u32(&done_bar), 0u, &no_abort)) ok = false;
-    }
-    // ------------------------------------------------------------- epilogue
-    if (warp < 4) {
-        // the MMA thread commits done_bar on every path, so this wait ends
-        // once its MMAs have landed (abort only shortens the error path)
-        const volatile int no_abort = 0;
-        const bool landed = mbar_wait_ws(smem_u32(&done_bar), 0u, &no_abort);
-        if (!landed) ok = false;
+        mma_commit_warp(smem_u32(&done_bar));
+        ok = __all_sync(0xffffffffu, mbar_wait_ws(smem_u32(&done_bar), 0u, &no_abort)) && ok;
+    } else {
+        // -------------------------------------- bias gradient, then epilogue
+        // thread: channels 8 (tid % NG) .. + 7 of the pixels tid / NG + 128 / NG i
+        constexpr int NG = CO / 8;
+        const int chb = tid % NG;
+        uint32_t jg = 0;
+        for (WsRows piece = ws_rows(rows); piece.at < piece.end && ok;) {
+            const WsItem it = ws_next(piece, segs, H);
+            for (int r = it.y0; r < it.y1; ++r, ++jg) {
+                const uint32_t s = jg % kWgGSlots;
+                ok = __all_sync(0xffffffffu, mbar_wait_ws(smem_u32(&gfull[s]),
+                                                          (jg / kWgGSlots) & 1u, &s_abort, lim));
+                if (!ok) break;
+                const uint8_t* slot = gring + s * S::kGRowBytes;
+#pragma unroll
+                for (int i = 0; i < NG; ++i) {
+                    const int p = tid / NG + i * (128 / NG);
+                    const int c = chb ^ (NG == 8 ? p & 7 : p >> 1 & 3);
+                    const uint4 v =
+                        *reinterpret_cast<const uint4*>(slot + p * S::kPitchG + c * 16);
+                    const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        bacc[2 * h] += __uint_as_float(e[h] << 16);
+                        bacc[2 * h + 1] += __uint_as_float(e[h] & 0xFFFF0000u);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&gempty[s]));
+            }
+        }
+        if (!ok) s_abort = 1;
+        // the MMA warp commits done_bar on every path, so this wait ends once
+        // its MMAs have landed
+        const bool landed =
+            __all_sync(0xffffffffu, mbar_wait_ws(smem_u32(&done_bar), 0u, &no_abort));
+        ok = ok && landed;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int L = warp * 32 + lane;  // TMEM lane = GEMM row
-        const int ci = L % CI, ri = L / CI;
+        const int L = warp * 32 + lane;  // TMEM lane
+        const int ci = L % CI;
         const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
         float* dst = part + (size_t)blockIdx.x * 9 * CO * CI;
 #pragma unroll
         for (int t = 0; t < S::kTiles; ++t) {
-            // tile t row ri is input row r - 1 + t + ri, i.e. dy index t + ri
-            const int dyi = t + ri;
-            const bool keep = landed && (S::kTiles == 2 ? (t == 0 || ri == 1) : ri < 3);
+            const int dx = 2 * t + L / CI;
 #pragma unroll
             for (int c0 = 0; c0 < S::kN; c0 += 32) {
                 uint32_t v[32];
                 tmem_ld32_raw(tmem + lane_off + (uint32_t)(t * S::kN + c0), v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (keep) {
+                if (landed && dx < 3) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
-                        const int n = c0 + j, dxi = n / CO, co = n % CO;
-                        dst[((size_t)(3 * dyi + dxi) * CO + co) * CI + ci] = __uint_as_float(v[j]);
+                        const int dy = 2 - (c0 + j) / CO, co = (c0 + j) % CO;
+                        dst[((size_t)(3 * dy + dx) * CO + co) * CI + ci] = __uint_as_float(v[j]);
                     }
                 }
             }
@@ -1422,12 +1456,12 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"((uint32_t)S::kTmemCols));
     }
-    // bias partial of the CTA: the producer threads of each channel chunk,
-    // in a fixed order
+    // bias partial of the CTA: the threads of each channel chunk, in a fixed
+    // order
     if (tid < CO) {
-        const int chb = tid / 8, k = tid % 8;
+        const int k = tid % 8;
         float t = 0.0f;
-        for (int q = chb; q < 128; q += NG) t += s_bias[q][k];
+        for (int q = tid / 8; q < 128; q += CO / 8) t += s_bias[q][k];
         partb[(size_t)blockIdx.x * CO + tid] = t;
     }
 }
@@ -1438,6 +1472,10 @@ hp_status launch_wgrad_t(const void* x, const void* gy, float* part, size_t part
                          int* grid_out, cudaStream_t st, uint32_t wait_limit)
 {
     using S = WgSmem<CI, CO>;
+    CUtensorMap xmap, gmap;
+    hp_status mrc = row_map(x, CI, W, H, B, kHaloPx, &xmap);
+    if (mrc == HP_OK) mrc = row_map(gy, CO, W, H, B, kTileM, &gmap);
+    if (mrc != HP_OK) return mrc;
     static bool attr = false;
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc_kernel<CI, CO>,
@@ -1447,17 +1485,12 @@ hp_status launch_wgrad_t(const void* x, const void* gy, float* part, size_t part
     }
     const int segs = (W + kTileM - 1) / kTileM;
     const long rows = (long)B * H * segs;
-    int band = (int)((rows + 4L * nsm - 1) / (4L * nsm));
-    band = band < 2 ? 2 : band > H ? H : band;
-    const int nbands = (H + band - 1) / band;
-    const long items = (long)B * segs * nbands;
-    if (items > 0x7fffffffL) return HP_ERR_INVALID_ARG;
-    const int grid = items < nsm ? (int)items : nsm;
+    if (rows > 0x7fffffffL) return HP_ERR_INVALID_ARG;
+    const int grid = rows < nsm ? (int)rows : nsm;
     if ((size_t)grid * 9 * CO * CI > part_len || (size_t)grid * CO > partb_len)
         return HP_ERR_INVALID_ARG;
     conv3x3_wgrad_tc_kernel<CI, CO><<<grid, kWgThreads, S::kBytes, st>>>(
-        (const uint4*)x, (const uint4*)gy, part, partb, H, W, segs, nbands, band, (int)items, err,
-        wait_limit);
+        part, partb, H, W, segs, (int)rows, err, wait_limit, xmap, gmap);
     *grid_out = grid;
     return check_launch();
 }
