@@ -23,12 +23,137 @@ namespace hp {
 
 namespace {
 
-struct Field {
-    const float* q;  // [My][Mx]
-    int Mx, My;
-    float ox, oy;    // position of sample (0, 0)
-    __device__ float at(int i, int j) const { return __ldg(q + (size_t)j * Mx + i); }
+// The four samples around a position.
+struct Corners {
+    float q00, q01, q10, q11;
 };
+
+// Mx x My samples, sample (0, 0) at (ox, oy).
+struct Field {
+    const float* q;
+    int Mx, My;
+    float ox, oy;
+    __device__ float at(int i, int j) const { return __ldg(q + (size_t)j * Mx + i); }
+    // samples (i, j) and its right and lower neighbours (itself where the
+    // field has one column or row)
+    __device__ Corners corners(int i, int j) const
+    {
+        const float* p = q + ((size_t)j * Mx + i);
+        const int di = Mx > 1 ? 1 : 0;
+        const float* r = p + (My > 1 ? Mx : 0);
+        return {__ldg(p), __ldg(p + di), __ldg(r), __ldg(r + di)};
+    }
+};
+
+// Density with the inlet applied: rho_in on the inlet cells.
+struct Rho {
+    const float* q;
+    int Mx, My;
+    float ox, oy;
+    int x0, x1;
+    float rho_in;
+    __device__ bool inlet(int i, int j) const { return j == My - 1 && i >= x0 && i < x1; }
+    __device__ float at(int i, int j) const
+    {
+        return inlet(i, j) ? rho_in : __ldg(q + (size_t)j * Mx + i);
+    }
+    __device__ Corners corners(int i, int j) const
+    {
+        Corners c = Field{q, Mx, My, ox, oy}.corners(i, j);
+        if (j + 2 >= My) {  // the lower row is the last one
+            const int i1 = min(i + 1, Mx - 1), j1 = min(j + 1, My - 1);
+            if (inlet(i, j)) c.q00 = rho_in;
+            if (inlet(i1, j)) c.q01 = rho_in;
+            if (inlet(i, j1)) c.q10 = rho_in;
+            if (inlet(i1, j1)) c.q11 = rho_in;
+        }
+        return c;
+    }
+};
+
+// Position along one axis: the sample at or below it and the distance to it.
+//
+// WIDE: fields of 2^22 samples and more along a row.  Else every coordinate
+// t and index lies in [0, 2^23), where FP32 addition of 2^23 leaves the whole
+// part in the low mantissa bits (rounded down), so that floor and both
+// conversions are plain additions.  The conversion instructions issue at an
+// eighth of their rate and six per sample held the step back.
+constexpr float kTwo23 = 8388608.0f;
+
+template <bool WIDE>
+__device__ __forceinline__ float to_float(int i)  // i >= 0
+{
+    if constexpr (WIDE) return (float)i;
+    else return __int_as_float(__float_as_int(kTwo23) + i) - kTwo23;
+}
+
+// t in [0, n - 1]; the last sample counts as distance 1 from the one before
+template <bool WIDE>
+__device__ __forceinline__ int split(float t, int n, float& frac)
+{
+    const int last = max(n - 2, 0);
+    if constexpr (WIDE) {
+        const int i = min((int)floorf(t), last);
+        frac = t - (float)i;
+        return i;
+    } else {
+        const float r = fminf(__fadd_rd(t, kTwo23), kTwo23 + (float)last);
+        frac = t - (r - kTwo23);
+        return __float_as_int(r) - __float_as_int(kTwo23);
+    }
+}
+
+struct Pos {
+    int i, j;
+    float fx, fy;
+};
+
+// (x, y) clamped to the sample span of f
+template <bool WIDE, class Q>
+__device__ __forceinline__ Pos locate(const Q& f, float x, float y)
+{
+    const float tx = fminf(fmaxf(x - f.ox, 0.0f), (float)(f.Mx - 1));
+    const float ty = fminf(fmaxf(y - f.oy, 0.0f), (float)(f.My - 1));
+    Pos p;
+    p.i = split<WIDE>(tx, f.Mx, p.fx);
+    p.j = split<WIDE>(ty, f.My, p.fy);
+    return p;
+}
+
+// Which product of a weighted sum goes unrounded into the fused addition, for
+// the top, the bottom and the vertical interpolation: written out, so that the
+// roundings do not depend on what a compiler makes of the code around them (a
+// projection's convergence amplifies the last bit of u* to 5e-6 in E_1).
+enum Fuse : bool { kFirst = true, kSecond = false };
+
+template <Fuse F>
+__device__ __forceinline__ float mix(float a, float wa, float b, float wb)
+{
+    return F == kFirst ? __fmaf_rn(a, wa, __fmul_rn(b, wb)) : __fmaf_rn(b, wb, __fmul_rn(a, wa));
+}
+
+template <Fuse TOP, Fuse BOT, Fuse VERT>
+__device__ __forceinline__ float blend(const Corners& c, const Pos& p)
+{
+    const float top = mix<TOP>(c.q00, 1.0f - p.fx, c.q01, p.fx);
+    const float bot = mix<BOT>(c.q10, 1.0f - p.fx, c.q11, p.fx);
+    return mix<VERT>(top, 1.0f - p.fy, bot, p.fy);
+}
+
+// The forward value of a quantity: density (kind 0), u (1) or v (2); OWN: as
+// a sample's own new value, else as MacCormack's forward field.
+template <bool MC, int KIND, bool OWN>
+__device__ __forceinline__ float blend_forward(const Corners& c, const Pos& p)
+{
+    if constexpr (KIND == 0) {
+        return MC ? blend<kFirst, kFirst, kFirst>(c, p) : blend<kFirst, kSecond, kFirst>(c, p);
+    } else if constexpr (KIND == 1) {
+        return MC && OWN ? blend<kSecond, kSecond, kFirst>(c, p)
+                         : blend<kSecond, kSecond, kSecond>(c, p);
+    } else {
+        return blend<kSecond, kSecond, kFirst>(c, p);
+    }
+}
 
 // Velocity at sample (i, j) of a quantity whose samples sit at (i + ox,
 // j + oy): cell centres (1/2, 1/2), u faces (0, 1/2) or v faces (1/2, 0).
@@ -65,126 +190,22 @@ __device__ __forceinline__ void vel_at_sample(const Field& fu, const Field& fv, 
     }
 }
 
-// Density field with the inlet applied: rho_in on the inlet cells.
-struct Rho {
-    const float* q;
-    int nx, ny, x0, x1;
-    float rho_in;
-    __device__ float at(int i, int j) const
-    {
-        return (j == ny - 1 && i >= x0 && i < x1) ? rho_in : __ldg(q + (size_t)j * nx + i);
-    }
-};
-
-// Generic quantity view: Mx x My samples, sample (0, 0) at (ox, oy).
-template <class Q>
-struct View {
-    const Q& q;
-    int Mx, My;
-    float ox, oy;
-};
-
-// Bilinear sample of a view at (x, y) (position clamped to the sample span),
-// with the range of the four samples it interpolates.
-template <class V>
-__device__ __forceinline__ float sample_range(const V& f, float x, float y, float* lo, float* hi)
+// Departure point of sample (i, j) of q and the samples around it, with the
+// velocity at (i, j).
+template <bool WIDE, class Q>
+__device__ __forceinline__ Pos departure(const Q& q, const Field& fu, const Field& fv, float dt,
+                                         int i, int j, float& vx, float& vy, Corners& c)
 {
-    const float tx = fminf(fmaxf(x - f.ox, 0.0f), (float)(f.Mx - 1));
-    const float ty = fminf(fmaxf(y - f.oy, 0.0f), (float)(f.My - 1));
-    int i0 = (int)floorf(tx), j0 = (int)floorf(ty);
-    i0 = min(i0, max(f.Mx - 2, 0));
-    j0 = min(j0, max(f.My - 2, 0));
-    const float fx = tx - (float)i0, fy = ty - (float)j0;
-    const int i1 = min(i0 + 1, f.Mx - 1), j1 = min(j0 + 1, f.My - 1);
-    const float q00 = f.q.at(i0, j0), q01 = f.q.at(i1, j0);
-    const float q10 = f.q.at(i0, j1), q11 = f.q.at(i1, j1);
-    if (lo) {
-        *lo = fminf(fminf(q00, q01), fminf(q10, q11));
-        *hi = fmaxf(fmaxf(q00, q01), fmaxf(q10, q11));
-    }
-    const float top = q00 * (1.0f - fx) + q01 * fx;
-    const float bot = q10 * (1.0f - fx) + q11 * fx;
-    return top * (1.0f - fy) + bot * fy;
-}
-
-// The forward semi-Lagrangian field of a quantity, evaluated on demand at
-// its own samples.
-template <class Q>
-struct Forward {
-    const Q& q;
-    const Field& fu;
-    const Field& fv;
-    int Mx, My;
-    float ox, oy, dt;
-    // the forward value at sample (i, j), with the velocity (vx, vy) there
-    __device__ float at_vel(int i, int j, float& vx, float& vy) const
-    {
-        const float x = (float)i + ox, y = (float)j + oy;
-        vel_at_sample(fu, fv, ox, oy, i, j, vx, vy);
-        const View<Q> w = {q, Mx, My, ox, oy};
-        return sample_range(w, x - dt * vx, y - dt * vy, nullptr, nullptr);
-    }
-    __device__ float at(int i, int j) const
-    {
-        float vx, vy;
-        return at_vel(i, j, vx, vy);
-    }
-};
-
-// New value of sample (i, j) of quantity q (Mx x My samples at (ox, oy)).
-template <bool MC, class Q>
-__device__ __forceinline__ float advected(const Q& q, int Mx, int My, float ox, float oy,
-                                          const Field& fu, const Field& fv, float dt, int i,
-                                          int j)
-{
-    const float x = (float)i + ox, y = (float)j + oy;
-    float vx, vy;
-    vel_at_sample(fu, fv, ox, oy, i, j, vx, vy);
-    const View<Q> w = {q, Mx, My, ox, oy};
-    if constexpr (!MC) {
-        return sample_range(w, x - dt * vx, y - dt * vy, nullptr, nullptr);
-    } else {
-        float lo, hi;
-        const float qf = sample_range(w, x - dt * vx, y - dt * vy, &lo, &hi);
-        const Forward<Q> fwd = {q, fu, fv, Mx, My, ox, oy, dt};
-        const View<Forward<Q>> wf = {fwd, Mx, My, ox, oy};
-        const float qb = sample_range(wf, x + dt * vx, y + dt * vy, nullptr, nullptr);
-        return fminf(fmaxf(qf + 0.5f * (q.at(i, j) - qb), lo), hi);
-    }
-}
-
-__device__ __forceinline__ float sample_rho(const Rho& r, float x, float y)
-{
-    const float tx = fminf(fmaxf(x - 0.5f, 0.0f), (float)(r.nx - 1));
-    const float ty = fminf(fmaxf(y - 0.5f, 0.0f), (float)(r.ny - 1));
-    int i0 = (int)floorf(tx), j0 = (int)floorf(ty);
-    i0 = min(i0, max(r.nx - 2, 0));
-    j0 = min(j0, max(r.ny - 2, 0));
-    const float fx = tx - (float)i0, fy = ty - (float)j0;
-    const int i1 = min(i0 + 1, r.nx - 1), j1 = min(j0 + 1, r.ny - 1);
-    const float top = r.at(i0, j0) * (1.0f - fx) + r.at(i1, j0) * fx;
-    const float bot = r.at(i0, j1) * (1.0f - fx) + r.at(i1, j1) * fx;
-    return top * (1.0f - fy) + bot * fy;
+    const float x = to_float<WIDE>(i) + q.ox, y = to_float<WIDE>(j) + q.oy;
+    vel_at_sample(fu, fv, q.ox, q.oy, i, j, vx, vy);
+    const Pos p = locate<WIDE>(q, x - dt * vx, y - dt * vy);
+    c = q.corners(p.i, p.j);
+    return p;
 }
 
 __device__ __forceinline__ bool fluid(const uint8_t* fl, int nx, int i, int j)
 {
     return fl[(size_t)j * nx + i] == 0;
-}
-
-// New density of cell (i, j).
-template <bool MC>
-__device__ __forceinline__ float rho_new_at(const Rho& r, const Field& fu, const Field& fv,
-                                            float dt, int i, int j)
-{
-    if constexpr (!MC) {
-        const float x = i + 0.5f, y = j + 0.5f;
-        float vx, vy;
-        vel_at_sample(fu, fv, 0.5f, 0.5f, i, j, vx, vy);
-        return sample_rho(r, x - dt * vx, y - dt * vy);
-    } else {
-        return advected<true>(r, r.nx, r.ny, 0.5f, 0.5f, fu, fv, dt, i, j);
-    }
 }
 
 // Tiles of the fused step: a CTA produces the outputs of kAdvTX x adv_ty(MC)
@@ -204,110 +225,129 @@ __host__ __device__ constexpr int adv_ty(bool mc) { return mc ? 16 : 32; }
 constexpr int kFW = kAdvTX + 2 * kAdvH;          // columns of a forward-field window
 constexpr int kFH = adv_ty(true) + 2 * kAdvH + 1;  // rows: tile rows - 1 - kAdvH .. + kAdvH
 
-// Forward field of quantity Q on its window (sample (ci, cj) at entry 0),
-// evaluated where it is not in the window.
-template <class Q>
-struct WindowedForward {
-    Forward<Q> f;
-    const float* s;
-    int ci, cj;
-    __device__ float at(int i, int j) const
-    {
-        const int a = i - ci, b = j - cj;
-        if (a >= 0 && a < kFW && b >= 0 && b < kFH) return s[b * kFW + a];
-        return f.at(i, j);
-    }
+constexpr int kFS = kFH * kFW;
+constexpr int kTS = (adv_ty(true) + 1) * kAdvTX;  // the tile and the row above it
+
+// What MacCormack's second half needs of a quantity: the forward field and the
+// velocity on the window (sample (ci, cj) at entry 0); on the tile, the value
+// itself and the range of the samples that it interpolates.
+struct Window {
+    float fwd[kFS], vx[kFS], vy[kFS];
+    float own[kTS], lo[kTS], hi[kTS];
 };
 
-// Fills the window of quantity q (Mx x My samples at (ox, oy)) with the
-// forward values and the velocities at the samples: the samples of the field
-// only (entries outside it are never read: every corner of a bilinear sample
-// lies in the field, and so does every output sample).
-template <class Q>
-__device__ __forceinline__ void fill_window(float* s, float* svx, float* svy, const Forward<Q>& f,
-                                            int ci, int cj)
+// Samples of the field only: entries outside it are never read (every corner
+// of a bilinear sample lies in the field, and so does every output sample).
+template <int KIND, bool WIDE, class Q>
+__device__ __forceinline__ void fill_entry(Window& w, const Q& q, const Field& fu, const Field& fv,
+                                           float dt, int a, int b, int ci, int cj)
 {
-    for (int t = threadIdx.x; t < kFH * kFW; t += kAdvThreads) {
-        const int b = t / kFW, a = t - b * kFW;
-        const int i = ci + a, j = cj + b;
-        if (i >= 0 && i < f.Mx && j >= 0 && j < f.My) {
-            float vx, vy;
-            s[t] = f.at_vel(i, j, vx, vy);
-            svx[t] = vx;
-            svy[t] = vy;
-        }
+    const int i = ci + a, j = cj + b;
+    if (i < 0 || i >= q.Mx || j < 0 || j >= q.My) return;
+    const int t = b * kFW + a;
+    float vx, vy;
+    Corners c;
+    const Pos p = departure<WIDE>(q, fu, fv, dt, i, j, vx, vy, c);
+    w.fwd[t] = blend_forward<true, KIND, false>(c, p);
+    w.vx[t] = vx;
+    w.vy[t] = vy;
+    const int ta = a - kAdvH, tb = b - kAdvH;
+    if ((unsigned)ta < (unsigned)kAdvTX && (unsigned)tb <= (unsigned)adv_ty(true)) {
+        const int tt = tb * kAdvTX + ta;
+        w.own[tt] = blend_forward<true, KIND, true>(c, p);
+        w.lo[tt] = fminf(fminf(c.q00, c.q01), fminf(c.q10, c.q11));
+        w.hi[tt] = fmaxf(fmaxf(c.q00, c.q01), fmaxf(c.q10, c.q11));
     }
 }
 
-// New value of sample (i, j) of quantity q: as advected<MC>, MacCormack's
-// backward sample and the velocity at (i, j) taken from the window.
-template <bool MC, class Q>
-__device__ __forceinline__ float advected_w(const Q& q, int Mx, int My, float ox, float oy,
-                                            const Field& fu, const Field& fv, float dt,
-                                            const float* win, const float* wvx,
-                                            const float* wvy, int ci, int cj, int i, int j)
+// New value of sample (i, j) of quantity q, in the first-order scheme the
+// forward value; in MacCormack's the backward sample reads the forward field
+// in the window, or evaluates the corners there that the window does not hold.
+template <bool MC, int KIND, bool WIDE, class Q>
+__device__ __forceinline__ float advected(const Window* w, const Q& q, const Field& fu,
+                                          const Field& fv, float dt, int ci, int cj, int i, int j)
 {
+    float vx, vy;
+    Corners c;
     if constexpr (!MC) {
-        return advected<false>(q, Mx, My, ox, oy, fu, fv, dt, i, j);
+        const Pos p = departure<WIDE>(q, fu, fv, dt, i, j, vx, vy, c);
+        return blend_forward<false, KIND, true>(c, p);
     } else {
-        const float x = (float)i + ox, y = (float)j + oy;
         const int t = (j - cj) * kFW + (i - ci);
-        const float vx = wvx[t], vy = wvy[t];
-        const View<Q> w = {q, Mx, My, ox, oy};
-        float lo, hi;
-        const float qf = sample_range(w, x - dt * vx, y - dt * vy, &lo, &hi);
-        const WindowedForward<Q> fwd = {{q, fu, fv, Mx, My, ox, oy, dt}, win, ci, cj};
-        const View<WindowedForward<Q>> wf = {fwd, Mx, My, ox, oy};
-        const float qb = sample_range(wf, x + dt * vx, y + dt * vy, nullptr, nullptr);
-        return fminf(fmaxf(qf + 0.5f * (q.at(i, j) - qb), lo), hi);
+        const int tt = (j - cj - kAdvH) * kAdvTX + (i - ci - kAdvH);
+        const float x = to_float<WIDE>(i) + q.ox, y = to_float<WIDE>(j) + q.oy;
+        const Pos p = locate<WIDE>(q, x + dt * w->vx[t], y + dt * w->vy[t]);
+        const int di = q.Mx > 1 ? 1 : 0, dj = q.My > 1 ? 1 : 0;
+        const int a = p.i - ci, b = p.j - cj;
+        if ((unsigned)a < (unsigned)(kFW - 1) && (unsigned)b < (unsigned)(kFH - 1)) {
+            const float* f = w->fwd + b * kFW + a;
+            c = {f[0], f[di], f[dj * kFW], f[dj * kFW + di]};
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < 4; ++k) {
+                const int ka = a + (k & 1) * di, kb = b + (k >> 1) * dj;
+                float val;
+                if ((unsigned)ka < (unsigned)kFW && (unsigned)kb < (unsigned)kFH) {
+                    val = w->fwd[kb * kFW + ka];
+                } else {
+                    Corners far;
+                    const Pos pf = departure<WIDE>(q, fu, fv, dt, ci + ka, cj + kb, vx, vy, far);
+                    val = blend_forward<true, KIND, false>(far, pf);
+                }
+                if (k == 0) c.q00 = val;
+                else if (k == 1) c.q01 = val;
+                else if (k == 2) c.q10 = val;
+                else c.q11 = val;
+            }
+        }
+        const float qb = blend<kFirst, kFirst, kFirst>(c, p);
+        return fminf(fmaxf(w->own[tt] + 0.5f * (q.at(i, j) - qb), w->lo[tt]), w->hi[tt]);
     }
 }
 
-// One CTA per tile: (MacCormack) the three forward-field windows; the new
-// density of the tile's rows and the row above, kept in shared memory for
-// the buoyancy; then the u and v faces.
-template <bool MC>
+// One CTA per tile: (MacCormack) the three windows; the new density of the
+// tile's rows and the row above, kept in shared memory for the buoyancy; then
+// the u and v faces.
+//
+// What bounds it: instruction issue.  MacCormack at 16 x 512^2 takes 158 us
+// (16 us of memory traffic); 187 us with the corners of every sample addressed
+// and clamped one by one, conversion instructions for the whole parts, and the
+// tile's own forward values and ranges interpolated a second time.
+template <bool MC, bool WIDE>
 __global__ void __launch_bounds__(kAdvThreads) advect_kernel(
     const float* __restrict__ u, const float* __restrict__ v, const float* __restrict__ rho,
     const uint8_t* __restrict__ flags, float* __restrict__ u_out, float* __restrict__ v_out,
     float* __restrict__ rho_out, int ny, int nx, hp_plume_params p)
 {
-    // forward rho, u, v and the velocity at their samples
-    __shared__ float s_win[MC ? 3 : 1][MC ? kFH * kFW : 1];
-    __shared__ float s_vx[MC ? 3 : 1][MC ? kFH * kFW : 1];
-    __shared__ float s_vy[MC ? 3 : 1][MC ? kFH * kFW : 1];
     constexpr int kAdvTY = adv_ty(MC);
     __shared__ float s_rho[(kAdvTY + 1) * kAdvTX];  // new rho, rows j0 - 1 ..
     const int i0 = blockIdx.x * kAdvTX, j0 = blockIdx.y * kAdvTY, b = blockIdx.z;
     const size_t cells = (size_t)ny * nx;
     const Field fu = {u + (size_t)b * ny * (nx + 1), nx + 1, ny, 0.0f, 0.5f};
     const Field fv = {v + (size_t)b * (ny + 1) * nx, nx, ny + 1, 0.5f, 0.0f};
-    const Rho r = {rho + b * cells, nx, ny, p.inlet_x0, p.inlet_x1, p.rho_in};
+    const Rho r = {rho + b * cells, nx, ny, 0.5f, 0.5f, p.inlet_x0, p.inlet_x1, p.rho_in};
     const uint8_t* fl = flags + b * cells;
     const float dt = p.dt;
     const int ci = i0 - kAdvH, cj = j0 - 1 - kAdvH;  // sample at entry 0 of a window
+    const Window* win[3] = {nullptr, nullptr, nullptr};
 
     if constexpr (MC) {
-        fill_window(s_win[0], s_vx[0], s_vy[0], Forward<Rho>{r, fu, fv, nx, ny, 0.5f, 0.5f, dt},
-                    ci, cj);
-        fill_window(s_win[1], s_vx[1], s_vy[1],
-                    Forward<Field>{fu, fu, fv, nx + 1, ny, 0.0f, 0.5f, dt}, ci, cj);
-        fill_window(s_win[2], s_vx[2], s_vy[2],
-                    Forward<Field>{fv, fu, fv, nx, ny + 1, 0.5f, 0.0f, dt}, ci, cj);
+        __shared__ Window s_win[3];  // rho, u, v
+        for (int t = threadIdx.x; t < kFS; t += kAdvThreads) {
+            const int wb = t / kFW, wa = t - wb * kFW;
+            fill_entry<0, WIDE>(s_win[0], r, fu, fv, dt, wa, wb, ci, cj);
+            fill_entry<1, WIDE>(s_win[1], fu, fu, fv, dt, wa, wb, ci, cj);
+            fill_entry<2, WIDE>(s_win[2], fv, fu, fv, dt, wa, wb, ci, cj);
+        }
+        for (int k = 0; k < 3; ++k) win[k] = &s_win[k];
         __syncthreads();
     }
-    constexpr int kU = MC ? 1 : 0, kV = MC ? 2 : 0;
 
     for (int t = threadIdx.x; t < (kAdvTY + 1) * kAdvTX; t += kAdvThreads) {
         const int rr = t / kAdvTX, c = t - rr * kAdvTX;
         const int i = i0 + c, j = j0 - 1 + rr;
         if (i < nx && j >= 0 && j < ny) {
-            float val;
-            if constexpr (MC)
-                val = advected_w<true>(r, nx, ny, 0.5f, 0.5f, fu, fv, dt, s_win[0], s_vx[0],
-                                       s_vy[0], ci, cj, i, j);
-            else
-                val = rho_new_at<false>(r, fu, fv, dt, i, j);
+            const float val = advected<MC, 0, WIDE>(win[0], r, fu, fv, dt, ci, cj, i, j);
             s_rho[t] = val;
             if (rr > 0) rho_out[b * cells + (size_t)j * nx + i] = val;
         }
@@ -321,9 +361,7 @@ __global__ void __launch_bounds__(kAdvThreads) advect_kernel(
         if (j < ny) {
             const bool open = i > 0 && i < nx && fluid(fl, nx, i - 1, j) && fluid(fl, nx, i, j);
             float val = 0.0f;
-            if (open)
-                val = advected_w<MC>(fu, nx + 1, ny, 0.0f, 0.5f, fu, fv, dt, s_win[kU], s_vx[kU],
-                                     s_vy[kU], ci, cj, i, j);
+            if (open) val = advected<MC, 1, WIDE>(win[1], fu, fu, fv, dt, ci, cj, i, j);
             u_out[(size_t)b * ny * (nx + 1) + (size_t)j * (nx + 1) + i] = val;
         }
         if (i < nx) {
@@ -331,9 +369,7 @@ __global__ void __launch_bounds__(kAdvThreads) advect_kernel(
             // an open top keeps (advects) its faces; buoyancy acts on interior faces
             const bool top = j == 0 && p.open_top && fluid(fl, nx, i, 0);
             float val = 0.0f;
-            if (interior || top)
-                val = advected_w<MC>(fv, nx, ny + 1, 0.5f, 0.0f, fu, fv, dt, s_win[kV], s_vx[kV],
-                                     s_vy[kV], ci, cj, i, j);
+            if (interior || top) val = advected<MC, 2, WIDE>(win[2], fv, fu, fv, dt, ci, cj, i, j);
             if (interior) {
                 // new density of cells (i, j - 1) and (i, j): rows rr and rr + 1
                 const float rf = 0.5f * (s_rho[rr * kAdvTX + c] + s_rho[(rr + 1) * kAdvTX + c]);
@@ -411,12 +447,10 @@ hp_status launch_advect(const float* u, const float* v, const float* rho, const 
 {
     const int ty = adv_ty(p.scheme == 1);
     dim3 blk(kAdvThreads), grd((s.nx + 1 + kAdvTX - 1) / kAdvTX, (s.ny + ty) / ty, s.batch);
-    if (p.scheme == 1)
-        advect_kernel<true><<<grd, blk, 0, st>>>(u, v, rho, flags, u_out, v_out, rho_out, s.ny,
-                                                 s.nx, p);
-    else
-        advect_kernel<false><<<grd, blk, 0, st>>>(u, v, rho, flags, u_out, v_out, rho_out, s.ny,
-                                                  s.nx, p);
+    const bool wide = s.nx >= 1 << 22 || s.ny >= 1 << 22;
+    auto kernel = p.scheme == 1 ? (wide ? advect_kernel<true, true> : advect_kernel<true, false>)
+                                : (wide ? advect_kernel<false, true> : advect_kernel<false, false>);
+    kernel<<<grd, blk, 0, st>>>(u, v, rho, flags, u_out, v_out, rho_out, s.ny, s.nx, p);
     return check_launch();
 }
 
