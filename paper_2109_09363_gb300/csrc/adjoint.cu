@@ -23,17 +23,6 @@ __device__ __forceinline__ float inv_open(uint32_t m)
     return n == 4 ? 0.25f : n == 3 ? (1.0f / 3.0f) : n == 2 ? 0.5f : n == 1 ? 1.0f : 0.0f;
 }
 
-// sum of q over the open-face neighbours of cell c
-__device__ __forceinline__ float open_sum(const float* q, uint32_t m, size_t c, int nx)
-{
-    float s = 0.0f;
-    if (m & 1u) s += q[c - 1];
-    if (m & 2u) s += q[c + 1];
-    if (m & 4u) s += q[c - nx];
-    if (m & 8u) s += q[c + nx];
-    return s;
-}
-
 // lam_k = D(g) + scale * g_p; mu_k = lam_k / n (k > 0) or g_phi0 = lam_k (k = 0)
 __global__ void adj_init_kernel(const float* __restrict__ gu, const float* __restrict__ gv,
                                 const float* __restrict__ gp, const uint8_t* __restrict__ mask,
@@ -56,24 +45,90 @@ __global__ void adj_init_kernel(const float* __restrict__ gu, const float* __res
     if (gp) lam += scale * gp[q];
     if (!(m & 15u)) lam = 0.0f;
     mu[q] = k > 0 ? lam * inv_open(m) : lam;
-    acc[q] = 0.0f;
+    if (k == 0) acc[q] = 0.0f;  // else written by the first block of sweeps
 }
 
-// acc += mu_t; mu_{t-1} = n^-1 W mu_t, or on the last step g_phi0 = W mu_1
-__global__ void adj_sweep_kernel(const float* __restrict__ mu_in, float* __restrict__ out,
-                                 float* __restrict__ acc, const uint8_t* __restrict__ mask,
-                                 int last, int ny, int nx)
+// A block of sweeps: acc += mu_t; mu_{t-1} = n^-1 W mu_t, and on the very last
+// sweep g_phi0 = W mu_1.
+//
+// One launch per sweep was bound by the launches; a block of 7 sweeps of
+// 8 x 256^2 takes 12.7 us (forward and backward of 20 sweeps, with what the
+// host takes for the call: 402 -> 377 us).
+// A CTA holds a region of kAdjN x kAdjN cells, each thread 8 rows of a column
+// in registers (mu, acc, 1/n, the face bits), so a sweep costs one shared store
+// and two shared loads per cell (west and east; north and south are the
+// thread's own) and one barrier.  A sweep makes one more ring of the region's
+// edge stale: with `sweeps` of them the outer hx columns and hy rows per side
+// (= sweeps, or 0 where the region holds the whole side of the grid) are
+// copies that other CTAs own.  kAdjSweeps = 8 keeps 48 x 48 of 64 x 64.
+constexpr int kAdjN = 64, kAdjRows = 8, kAdjThreads = kAdjN * (kAdjN / kAdjRows);
+constexpr int kAdjSweeps = 8;
+
+__global__ void __launch_bounds__(kAdjThreads, 2)
+    adj_block_kernel(const float* __restrict__ mu_in, float* __restrict__ out,
+                     float* __restrict__ acc, const uint8_t* __restrict__ mask, int sweeps, int hx,
+                     int hy, int first, int last, int ny, int nx)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    const int b = blockIdx.z;
-    if (i >= nx) return;
-    const size_t base = (size_t)b * ny * nx;
-    const size_t c = (size_t)j * nx + i;
-    const uint32_t m = mask[base + c];
-    acc[base + c] += mu_in[base + c];
-    const float s = open_sum(mu_in + base, m, c, nx);
-    out[base + c] = last ? s : s * inv_open(m);
+    __shared__ float s_mu[2][kAdjN + 2][kAdjN + 2];
+    const int lx = threadIdx.x % kAdjN, ly = threadIdx.x / kAdjN * kAdjRows;
+    const int x = blockIdx.x * (kAdjN - 2 * hx) - hx + lx;
+    const int y = blockIdx.y * (kAdjN - 2 * hy) - hy + ly;
+    const size_t base = (size_t)blockIdx.z * ny * nx;
+    // the ring around the region is read by its (stale) edge cells only
+    for (int i = threadIdx.x; i < 2 * (kAdjN + 2); i += kAdjThreads) {
+        const int h = i / (kAdjN + 2), c = i % (kAdjN + 2);
+        s_mu[h][0][c] = s_mu[h][kAdjN + 1][c] = s_mu[h][c][0] = s_mu[h][c][kAdjN + 1] = 0.0f;
+    }
+    const bool xin = x >= 0 && x < nx;
+    const bool xown = xin && lx >= hx && lx < kAdjN - hx;
+    float mu[kAdjRows], sum[kAdjRows], inv[kAdjRows];
+    uint32_t faces = 0u;  // four bits per row
+#pragma unroll
+    for (int k = 0; k < kAdjRows; ++k) {
+        const int j = y + k;
+        const bool in = xin && j >= 0 && j < ny;
+        const size_t q = base + (size_t)j * nx + x;
+        const uint32_t m = in ? mask[q] & 15u : 0u;
+        mu[k] = in ? mu_in[q] : 0.0f;
+        const bool own = xown && in && ly + k >= hy && ly + k < kAdjN - hy;
+        sum[k] = own && !first ? acc[q] : 0.0f;
+        inv[k] = inv_open(m);
+        faces |= m << (4 * k);
+    }
+    for (int t = 0; t < sweeps; ++t) {
+        // (unpacked in every sweep: hoisted, the face tests spill)
+        asm volatile("" : "+r"(faces));
+        float(*s)[kAdjN + 2] = s_mu[t & 1];
+#pragma unroll
+        for (int k = 0; k < kAdjRows; ++k) s[ly + k + 1][lx + 1] = mu[k];
+        __syncthreads();
+        const bool scaled = !(last && t == sweeps - 1);
+        float north = s[ly][lx + 1];
+        const float below = s[ly + kAdjRows + 1][lx + 1];
+#pragma unroll
+        for (int k = 0; k < kAdjRows; ++k) {
+            const uint32_t m = faces >> (4 * k);
+            const float west = s[ly + k + 1][lx], east = s[ly + k + 1][lx + 2];
+            const float south = k + 1 < kAdjRows ? mu[k + 1 < kAdjRows ? k + 1 : k] : below;
+            sum[k] += mu[k];
+            float w = 0.0f;
+            if (m & 1u) w += west;
+            if (m & 2u) w += east;
+            if (m & 4u) w += north;
+            if (m & 8u) w += south;
+            north = mu[k];
+            mu[k] = scaled ? w * inv[k] : w;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kAdjRows; ++k) {
+        const int j = y + k;
+        if (xown && j >= 0 && j < ny && ly + k >= hy && ly + k < kAdjN - hy) {
+            const size_t q = base + (size_t)j * nx + x;
+            out[q] = mu[k];
+            acc[q] = sum[k];
+        }
+    }
 }
 
 // g_u* = g_u + (acc_c - acc_nb) on open faces, 0 on closed faces
@@ -124,11 +179,20 @@ extern "C" hp_status hp_project_adjoint(hp_ctx* ctx, const float* gu, const floa
     adj_init_kernel<<<grd, blk, 0, st>>>(gu, gv, gp, ctx->mask, rho0 / dt, k > 0 ? bufs[0] : g_phi0,
                                          acc, k, s.ny, s.nx);
     if ((rc = check_launch()) != HP_OK) return rc;
-    for (int t = k; t >= 1; --t) {
-        const int cur = (k - t) & 1;
-        float* out = t == 1 ? g_phi0 : bufs[cur ^ 1];
-        adj_sweep_kernel<<<grd, blk, 0, st>>>(bufs[cur], out, acc, ctx->mask, t == 1, s.ny, s.nx);
+    // blocks of nearly equal length; a grid that one region holds takes one
+    const bool whole = s.nx <= kAdjN && s.ny <= kAdjN;
+    int left = k, cur = 0;
+    for (int n = k == 0 ? 0 : whole ? 1 : (k - 1) / kAdjSweeps + 1; n > 0; --n) {
+        const int sweeps = (left - 1) / n + 1;
+        const int hx = s.nx <= kAdjN ? 0 : sweeps, hy = s.ny <= kAdjN ? 0 : sweeps;
+        const int ox = kAdjN - 2 * hx, oy = kAdjN - 2 * hy;
+        const dim3 tiles((s.nx + ox - 1) / ox, (s.ny + oy - 1) / oy, s.batch);
+        adj_block_kernel<<<tiles, kAdjThreads, 0, st>>>(bufs[cur], n == 1 ? g_phi0 : bufs[cur ^ 1],
+                                                        acc, ctx->mask, sweeps, hx, hy, left == k,
+                                                        n == 1, s.ny, s.nx);
         if ((rc = check_launch()) != HP_OK) return rc;
+        left -= sweeps;
+        cur ^= 1;
     }
     adj_correct_kernel<<<grd, blk, 0, st>>>(gu, gv, acc, ctx->mask, gu_star, gv_star, s.ny, s.nx);
     return check_launch();
