@@ -1208,7 +1208,7 @@ def main():
                            use_graph=0 if args.host_loop else 1,
                            sweep_kernel=args.sweep_kernel)
     # the grid-resident kernel runs when the library picks it (0) or it is
-    # asked for (4) and one cluster per grid fits on this device
+    # asked for (4) and the SMs hold a grid of this shape
     resident = args.sweep_kernel in (0, 4) and hp.hp_resident_clusters(ctx, B, N, N) > 0
     streaming = not resident and streaming_chosen(args.sweep_kernel, B * N * N)
     per_launch = 1 if streaming else T_BLOCK
@@ -1227,8 +1227,8 @@ def main():
     torch.cuda.synchronize()
     iters = out["iters"].cpu().numpy()
     if resident:
-        # mask/div, init, reset, the resident sweep loop, correction, norms (2)
-        launches_per_step = 7
+        # mask/div, preparation, the resident sweep loop, correction, norms (2)
+        launches_per_step = 6
     elif streaming:
         # 8 sweep launches per graph-loop iteration, plus mask/div, init,
         # reset, correction, norms, finish
@@ -1315,7 +1315,7 @@ def main():
                                       "note": "13 B per cell-sweep of a sweep that streams "
                                               "from HBM; the resident kernel reads the grid "
                                               "once per projection"},
-                    "note": "one cluster of 16 CTAs per 512^2 grid keeps phi on chip for all "
+                    "note": "strips of a grid stay on chip, one SM each, for all "
                             "sweeps; per-sweep time of the 16-grid batch from two fixed-length "
                             "runs"}
     else:
@@ -1398,7 +1398,7 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": WORKLOAD, "method": "plain Jacobi", "grids_per_gpu": B,
                        "grid": [N, N], "threshold": THR, "cap": CAP,
-                       "sweep_kernel": ("grid-resident (one cluster per grid)" if resident
+                       "sweep_kernel": ("grid-resident (strips, one SM each)" if resident
                                         else "streaming" if streaming else "temporally blocked"),
                        "temporal_block": None if (streaming or resident) else T_BLOCK,
                        "loop": ("one launch per projection" if resident else "host-polled"
