@@ -1202,7 +1202,8 @@ hp_status hp_project_hybrid(hp_ctx* ctx, hp_cnn* cnn, float* u, float* v, const 
         !cnn_shape_ok(cnn, s))
         return HP_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    // divergence into the context, CNN guess into the first phi buffer
+    // divergence into the context, CNN guess into the second phi buffer
+    // (the sweeps write the first, and read cells of a guess that another CTA owns)
     hp_status rc = launch_mask_div(u, v, flags, ctx->mask, ctx->div, s, st, boundary_of(*prm));
     if (rc != HP_OK) return rc;
     float* phi_hat = cnn->out[cnn->br.n - 1];
@@ -1219,11 +1220,11 @@ hp_status hp_project_hybrid(hp_ctx* ctx, hp_cnn* cnn, float* u, float* v, const 
         phi_hat, cnn->s, ctx->mask, cnn->guess_bad, s.batch, cells);
     if ((rc = check_launch()) != HP_OK) return rc;
     phi0_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(phi_hat, cnn->s, ctx->mask,
-                                                             cnn->guess_bad, ctx->phi[0],
+                                                             cnn->guess_bad, ctx->phi[1],
                                                              cnn->err, s.batch, cells);
     if ((rc = check_launch()) != HP_OK) return rc;
     // the mask and divergence of the context are those of this velocity
-    return project_impl(ctx, u, v, flags, s, prm, ctx->phi[0], p_out, iters_out, e1_out,
+    return project_impl(ctx, u, v, flags, s, prm, ctx->phi[1], p_out, iters_out, e1_out,
                         einf_out, conv_out, e_hist, hist_len, st, nullptr, true);
 }
 

@@ -325,9 +325,9 @@ __global__ void reset_state_kernel(GridState* gs, LoopState* ls, int B)
     }
 }
 
-// phi_0 = given guess on cells with an open face, else 0 (out may be phi0).
-__global__ void init_phi_kernel(const float* phi0, const uint8_t* __restrict__ mask, float* out,
-                                size_t cells)
+// phi_0 = given guess on cells with an open face, else 0.
+__global__ void init_phi_kernel(const float* __restrict__ phi0, const uint8_t* __restrict__ mask,
+                                float* __restrict__ out, size_t cells)
 {
     const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= cells) return;

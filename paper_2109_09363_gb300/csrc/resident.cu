@@ -116,6 +116,7 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     *launched = false;
     ResPlan p;
     if (!res_plan(ctx, s, &p)) return HP_OK;
+    if (phi0 == ctx->phi[0]) return HP_ERR_INVALID_ARG;  // see ResArgs::phi
     const ResKernel k = res_kernel(p.width, p.R);
     cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
     cudaFuncAttributes fa;

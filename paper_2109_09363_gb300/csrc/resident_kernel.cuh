@@ -93,8 +93,13 @@ struct ResColumns {
 
 struct ResArgs {
     const float* phi0;  // phi_0 of the caller (cells without an open face ignored), null = 0
-    float* phi;         // phi_{k*} out (may be phi0)
-    float* ck[2];       // checkpoint buffers [B][ny][nx]
+    // phi_{k*} out, and phi at the cap as it passes: not phi0, since a strip with
+    // copied columns reads its neighbours' cells of phi_0 (again for a replay
+    // from it) when these may already be storing phi_{k*}
+    float* phi;
+    // checkpoint buffers [B][ny][nx]; phi0 may be ck[1], which is first written
+    // at sweep 64, when every strip has read phi_0 and no replay starts from it
+    float* ck[2];
     const float* div;   // [B][ny][nx]
     const uint8_t* mask;
     GridState* gs;
@@ -901,8 +906,6 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         int base = 0;  // the iterate that a replay would start from
         const float* from = a.phi0;
         if (with_e) {
-            // phi at the cap: not where a checkpoint it may still need lies
-            float* cap_buf = a.cap < 64 ? a.ck[1] : a.phi;
             int last = 0, before = 0, cb = 1;  // latest checkpoints, buffer of the latest
             // four sweeps at a time; round q needs the sums of sweeps 4q .. 4q+3,
             // the last stored during sweep 4q + 4
@@ -940,7 +943,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     float* wsum = s_wsum + ((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
                                   w.wid;
                     if (k + i <= a.cap) {
-                        if (k + i == a.cap) store_cells(cap_buf);
+                        if (k + i == a.cap) store_cells(a.phi);
                         w.template update<true>(phi, pending, wsum, a.err);
                     } else if (k + i - 1 == a.cap) {
                         // past the cap only its sum is left to do
@@ -960,11 +963,6 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             estar = sh.estar;
             first += (uint32_t)(k / 4 - 1);
             w.drain(a.err);
-            if (kstar == a.cap && cap_buf != a.phi) {
-                // each thread its own cells
-                load_cells(cap_buf, false, vec);
-                store_cells(a.phi);
-            }
             base = kstar >= last ? last : before;
             from = base == 0 ? a.phi0 : base == last ? a.ck[cb] : a.ck[cb ^ 1];
         }
