@@ -144,12 +144,15 @@ struct ResLayout {
     static_assert(kBytes <= 227 * 1024 - 64, "shared memory of one CTA");
 };
 
-// ---- 16-byte words through the L2 (each 8-byte half holds a value and its tag)
+// ---- 16-byte words through the L2: two 64-bit elements, each a value and its
+// tag.  A vector access promises nothing beyond its elements (PTX models it as
+// one access per element, in any order), so the pair has to be one element.
 
 __device__ __forceinline__ uint4 ld_box(const uint4* p)
 {
     uint4 v;
-    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("{\n\t.reg .b64 lo, hi;\n\tld.relaxed.gpu.global.v2.b64 {lo, hi}, [%4];\n\t"
+                 "mov.b64 {%0, %1}, lo;\n\tmov.b64 {%2, %3}, hi;\n\t}"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p)
                  : "memory");
@@ -158,8 +161,8 @@ __device__ __forceinline__ uint4 ld_box(const uint4* p)
 
 __device__ __forceinline__ void st_box(uint4* p, uint32_t a, uint32_t b, uint32_t tag)
 {
-    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a), "r"(tag),
-                 "r"(b), "r"(tag)
+    asm volatile("{\n\t.reg .b64 lo, hi;\n\tmov.b64 lo, {%1, %2};\n\tmov.b64 hi, {%3, %2};\n\t"
+                 "st.relaxed.gpu.global.v2.b64 [%0], {lo, hi};\n\t}" ::"l"(p), "r"(a), "r"(tag), "r"(b)
                  : "memory");
 }
 
