@@ -133,6 +133,12 @@ void hp_ctx_destroy(hp_ctx *ctx);
  * the last check (its results are then void), else HP_OK. */
 hp_status hp_ctx_check(hp_ctx *ctx);
 
+/* Polls after which a wait of the grid-resident sweeps gives up, for calls
+ * launched from now on; 0 = the compiled limits (about a second).  Its strips
+ * wait for one another's rows, and a wait can run out when the device runs
+ * some of them much later than the others. */
+hp_status hp_ctx_set_wait_limit(hp_ctx *ctx, uint32_t polls);
+
 const char *hp_status_string(hp_status s);
 const char *hp_last_cuda_error(void);
 

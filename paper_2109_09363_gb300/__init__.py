@@ -52,6 +52,7 @@ _SIGS = {
     "hp_ctx_create": (ctypes.c_int, [ctypes.POINTER(_P), hp_shape, ctypes.c_int]),
     "hp_ctx_destroy": (None, [_P]),
     "hp_ctx_check": (ctypes.c_int, [_P]),
+    "hp_ctx_set_wait_limit": (ctypes.c_int, [_P, ctypes.c_uint32]),
     "hp_trainer_check": (ctypes.c_int, [_P]),
     "hp_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "hp_last_cuda_error": (ctypes.c_char_p, []),
@@ -181,8 +182,14 @@ class Context:
 
     def check(self):
         """Raise if a kernel wrote into a guard zone past one of this
-        context's workspaces (synchronises the device)."""
+        context's workspaces, or if a wait of the grid-resident sweeps gave up
+        since the last check (synchronises the device)."""
         _check(load_library().hp_ctx_check(self._h))
+
+    def set_wait_limit(self, polls: int):
+        """Polls after which a wait of the grid-resident sweeps gives up (0:
+        the compiled limits)."""
+        _check(load_library().hp_ctx_set_wait_limit(self._h, int(polls)))
 
     def close(self):
         if self._h:

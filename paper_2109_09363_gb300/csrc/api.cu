@@ -230,6 +230,13 @@ hp_status hp_ctx_check(hp_ctx* c)
     return gave_up ? HP_ERR_TIMEOUT : HP_OK;
 }
 
+hp_status hp_ctx_set_wait_limit(hp_ctx* c, uint32_t polls)
+{
+    if (!c || polls > 0x7fffffffu) return HP_ERR_INVALID_ARG;
+    c->wait_limit = (int32_t)polls;
+    return HP_OK;
+}
+
 hp_status hp_face_mask(const uint8_t* flags, uint8_t* mask_out, hp_shape s, void* stream)
 {
     if (!flags || !mask_out || !shape_ok(s)) return HP_ERR_INVALID_ARG;

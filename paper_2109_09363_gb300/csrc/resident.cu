@@ -137,6 +137,8 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     a.cols = p.ntx > 1 ? (ResColumns*)ctx->cols : nullptr;
     a.ntx = p.ntx;
     a.err = ctx->wait_err;
+    a.polls = ctx->wait_limit ? ctx->wait_limit : kResPolls;
+    a.looks = ctx->wait_limit ? ctx->wait_limit : kResLooks;
     a.e_hist = e_hist;
     a.hist_len = hist_len;
     a.B = s.batch;

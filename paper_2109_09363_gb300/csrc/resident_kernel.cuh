@@ -64,9 +64,12 @@ static_assert(kResSweepers * kResRegsSweep + 128 * kResRegsHelp <= kResThreads *
 constexpr int kResLag = 3;
 constexpr int kResRing = 4;        // > kResLag: rounds between the sweeps and the decision
 constexpr int kWsumRing = 4 * kResRing;  // warp sums, by sweep
-// polls of a bounded wait before it gives up (each at least one L2 round
-// trip, so half a second or more); of a shared-memory wait
-constexpr int kResPolls = 1 << 20, kResSpins = 1 << 22;
+// A wait gives up after so many polls: of a word in the L2 (a round trip, half
+// a microsecond, so about a second) or of a barrier (suspended for a microsecond
+// at most); of a word in shared memory, which waits for a warp that waits for
+// the others.  The CTA then marks the launch, waits no longer than one poll
+// each for the rest of its grid (whose result is void) and takes no other grid.
+constexpr int kResPolls = 1 << 21, kResLooks = 1 << 27;
 // the sums of pairs are scaled (exactly) so that no sum of finite warp sums overflows
 constexpr float kSumScale = 1.0f / 4096.0f;
 static_assert(kResMaxCtas * kResWarps <= 4096, "warp sums of one grid");
@@ -106,6 +109,7 @@ struct ResArgs {
     ResBox* box;
     ResColumns* cols;   // null unless ntx > 1
     int32_t* err;       // set to 1 when a wait gave up
+    int32_t polls, looks;  // limits of the waits (kResPolls, kResLooks)
     double* e_hist;     // [B][hist_len] or null
     int32_t hist_len;
     int32_t B, ny, nx;
@@ -184,17 +188,17 @@ __device__ __forceinline__ void bar_arrive(uint64_t* b)
 }
 
 // whether the phase of this parity has completed; bounded
-__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, int spins)
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, int polls)
 {
     uint32_t done = 0;
     do {
         asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\t"
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(done)
-            : "r"(res_smem(b)), "r"(parity)
+            : "r"(res_smem(b)), "r"(parity), "r"(1000u)  // ns
             : "memory");
-    } while (!done && --spins > 0);
+    } while (!done && --polls > 0);
     return done != 0;
 }
 
@@ -235,6 +239,13 @@ __device__ __forceinline__ Pair pair_tree(Pair v)
     return v;
 }
 
+// A wait of this CTA ran out.
+__device__ __forceinline__ void give_up(const ResArgs& a, volatile int& lost)
+{
+    *a.err = 1;
+    lost = 1;
+}
+
 template <int C, int R, int WX>
 struct ResWarp {
     using L = ResLayout<C, R, WX>;
@@ -253,9 +264,10 @@ struct ResWarp {
     int out_r, out_c; // of this warp's own rows and column
     int in_h;         // of the row received from the neighbouring CTA
     uint64_t* full;   // [parity]: it is there
+    volatile int* lost;  // ResShared::lost
     uint4* tx;        // [parity][word] to the neighbouring CTA, this lane
     uint32_t t;       // messages sent (= received and being waited for) so far
-    bool dead;        // a wait gave up: do not wait any more
+    bool dead;        // a wait of this lane gave up: do not wait any more
 
     __device__ __forceinline__ void ld_row(int off, float (&v)[C]) const
     {
@@ -274,11 +286,11 @@ struct ResWarp {
     }
     static constexpr int kMsgLanes = 32 * WX;
     // the row of message t, from the helper that receives it; bounded
-    __device__ __forceinline__ void receive(float (&v)[C], int32_t* err)
+    __device__ __forceinline__ void receive(float (&v)[C], const ResArgs& a)
     {
-        if (!bar_wait(full + (t & 1u), (t - 1) >> 1 & 1u, dead ? 1 : kResSpins)) {
+        if (!bar_wait(full + (t & 1u), (t - 1) >> 1 & 1u, dead ? 1 : a.polls)) {
             dead = true;
-            *err = 1;
+            give_up(a, *lost);
         }
         ld_row(in_h + (t & 1u ? L::kHaloPar : 0), v);
     }
@@ -310,11 +322,11 @@ struct ResWarp {
         }
     }
     // every message is received, also the one no sweep uses: the sender counts on it
-    __device__ __forceinline__ void drain(int32_t* err)
+    __device__ __forceinline__ void drain(const ResArgs& a)
     {
         if (rem) {
             float v[C];
-            receive(v, err);
+            receive(v, a);
         }
     }
 
@@ -324,7 +336,7 @@ struct ResWarp {
     // 0, and becomes the sum of |r(phi_k)|.
     template <bool WITH_E>
     __device__ __forceinline__ void update(float (&phi)[R][C], float& pending, float* wsum,
-                                           int32_t* err)
+                                           const ResArgs& a)
     {
         const int pr = (t & 1u) ? L::kRowPar : 0, pc = (t & 1u) ? L::kColPar : 0;
         const int qr = L::kRowPar - pr, qc = L::kColPar - pc;
@@ -335,7 +347,7 @@ struct ResWarp {
         const bool far = (cls >> 16) != 0;
         // ds of the row before: south difference, the negated north one of this row
         float dsp[C];
-        if (far) receive(dsp, err);
+        if (far) receive(dsp, a);
         else ld_row(in_f + pr, dsp);
 #pragma unroll
         for (int q = 0; q < C; ++q) dsp[q] = __fsub_rn(phi[0][q], dsp[q]);
@@ -474,6 +486,7 @@ struct ResShared {
     int kstar, code;           // k*; 1 converged, 2 not
     double estar;
     int act;                   // 1: leave the sweep loop
+    volatile int lost;         // 1: a wait gave up
     int grid;                  // next grid of the group
 };
 
@@ -495,7 +508,7 @@ __device__ __forceinline__ void res_receiver(const ResArgs& a, uint8_t* sm, ResS
         for (int x = 0; x < WX; ++x) {
             const uint4* p = &a.box->row[cta][side][t & 1u][32 * x + lane];
             uint4 v[W];
-            int left = kResPolls;
+            int left = a.polls;
             for (;;) {
                 bool ok = true;
 #pragma unroll
@@ -507,7 +520,7 @@ __device__ __forceinline__ void res_receiver(const ResArgs& a, uint8_t* sm, ResS
                 const uint32_t end = sh.end;
                 if (__any_sync(0xffffffffu, end != 0 && t > end)) return;
                 if (--left <= 0) {
-                    *a.err = 1;
+                    give_up(a, sh.lost);
                     return;
                 }
             }
@@ -532,10 +545,9 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
     const double inv_cells = 1.0 / ((double)a.nx * (double)a.ny * kSumScale);
     for (int q = 0;; ++q) {
         const uint32_t e = first + q, tag = e + 1, slot = e % kResRing;
-        if (!bar_wait(&sh.sums[slot], e / kResRing & 1u, kResSpins)) {
-            *a.err = 1;
-            return;
-        }
+        // (lanes look at a barrier and at words one by one: every decision
+        // about a wait is taken by the warp)
+        bool there = __all_sync(0xffffffffu, bar_wait(&sh.sums[slot], e / kResRing & 1u, a.polls));
         const float* ws = s_wsum + (e * 4 + gi) % kWsumRing * kResWarps;
         Pair sum = pair_tree({ws[li] * kSumScale, 0.0f});
         if (n > 1) {
@@ -546,7 +558,7 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
                 sum = {0.0f, 0.0f};
                 for (int i = li; i < n; i += 32) {  // four loads in flight
                     uint4 v[4];
-                    int left = kResPolls;
+                    int left = there ? a.polls : 1;
                     bool ok;
                     do {
                         ok = true;
@@ -557,13 +569,13 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
                             ok = ok && v[u].y == tag && v[u].w == tag;
                         }
                     } while (!ok && --left > 0);
-                    if (left <= 0) *a.err = 1;
+                    there = there && ok;
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
                         if (i + 8 * u < n)
                             sum = pair_add(sum, {__uint_as_float(v[u].x), __uint_as_float(v[u].z)});
                 }
-                __syncwarp();
+                there = __all_sync(0xffffffffu, there);
                 sum = pair_tree(sum);
             }
         }
@@ -582,25 +594,22 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
             const int from = hit ? __ffs(hit) - 1 : 31;
             if (a.e_hist && li == 0 && lane <= from && j < a.hist_len)
                 a.e_hist[(size_t)b * a.hist_len + j] = ej;
-            code = __shfl_sync(0xffffffffu, c, from);
-            ks = 4 * q + (from >> 3);
+            code = there ? __shfl_sync(0xffffffffu, c, from) : 2;  // 2: all leave
+            ks = there ? 4 * q + (from >> 3) : 0;
             if (lane == from) sh.estar = ej;
             if (n > 1 && lane == 0)
                 st_box(&a.box->dec[group][slot], (uint32_t)code, (uint32_t)ks, tag);
         } else {
             uint4 v;
-            int left = kResPolls;
+            int left = there ? a.polls : 1;
             do {
                 v = ld_box(&a.box->dec[group][slot]);
             } while ((v.y != tag || v.w != tag) && --left > 0);
-            if (left <= 0) {
-                *a.err = 1;
-                v.x = 2;  // leave: the result of this call is void
-                v.z = 0;
-            }
-            code = (int)v.x;
-            ks = (int)v.z;
+            there = __all_sync(0xffffffffu, there && v.y == tag && v.w == tag);
+            code = there ? (int)v.x : 2;
+            ks = there ? (int)v.z : 0;
         }
+        if (!there) give_up(a, sh.lost);
         __syncwarp();
         if (lane == 0) {
             if (code != 0) {
@@ -623,12 +632,12 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
 template <int R, int WX>
 __device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float (&phi)[R][8],
                                             int cta, int wid, int lane, bool left, bool right,
-                                            uint32_t m, bool& dead)
+                                            uint32_t m, bool& dead, volatile int& lost)
 {
     using L = ResLayout<8, R, WX>;
     constexpr int W = R / 8;  // words per lane and side
     float* stage = reinterpret_cast<float*>(sm + L::kGhost) + wid * 2 * R * kResGhost;
-    __syncwarp();
+    dead = __any_sync(0xffffffffu, dead);  // the polls below are the warp's
     if (lane == 1 || lane == 30) {
         float4* dst = reinterpret_cast<float4*>(stage + (lane == 1 ? 0 : R * kResGhost));
 #pragma unroll
@@ -655,7 +664,7 @@ __device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float
         if (side ? !right : !left) continue;
         const uint4* box = a.cols->w[cta][side][m & 1u][wid][0];
         uint4 v[W];
-        int polls = dead ? 1 : kResPolls;
+        int polls = dead ? 1 : a.polls;
         for (;;) {
             bool ok = true;
 #pragma unroll
@@ -666,7 +675,7 @@ __device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float
             if (__all_sync(0xffffffffu, ok)) break;
             if (--polls <= 0) {
                 dead = true;
-                *a.err = 1;
+                give_up(a, lost);
                 break;
             }
         }
@@ -723,6 +732,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             for (int i = 0; i < 4; ++i) bar_init(&sh.full[i / 2][i % 2], 1);
             for (int i = 0; i < kResRing; ++i) bar_init(&sh.sums[i], kResWarps);
             sh.end = 0u;
+            sh.lost = 0;
         }
     }
     __syncthreads();
@@ -769,6 +779,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
     }
     w.t = 0;
     w.dead = false;
+    w.lost = &sh.lost;
     const bool left = WIDE && tx > 0, right = WIDE && tx < ntx - 1;
     const int x0 = (WIDE ? tx * (32 * C - 2 * kResGhost) - kResGhost : 0) + (w.wx * 32 + w.lane) * C;
     const int y0 = (ty * L::WY + w.wy) * R;
@@ -855,7 +866,8 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         auto refresh = [&]() {
             if constexpr (WIDE) {
                 ++fetched;
-                res_columns<R, WX>(a, sm, phi, cta, w.wid, w.lane, left, right, fetched, w.dead);
+                res_columns<R, WX>(a, sm, phi, cta, w.wid, w.lane, left, right, fetched, w.dead,
+                                   sh.lost);
                 w.publish(phi);
                 sync_sweepers();
             }
@@ -922,7 +934,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     last = k;
                 }
                 if (WIDE && k > 0 && k % kResGhost == 0 && k <= a.cap) {
-                    w.drain(a.err);
+                    w.drain(a);
                     refresh();
                 }
 #pragma unroll 1
@@ -930,11 +942,11 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     if (i == 2 && threadIdx.x == 0 && k + 4 >= 4 * kResLag) {
                         // the decision of round k / 4 + 1 - kResLag: long there
                         const int q = k / 4 + 1 - kResLag;
-                        int left = kResSpins;
+                        int left = a.looks;
                         while (sh.rounds <= q && --left > 0) {
                         }
-                        if (left <= 0) {
-                            *a.err = 1;
+                        if (sh.rounds <= q) {
+                            give_up(a, sh.lost);
                             sh.kstar = 0;
                             sh.code = 2;
                             sh.estar = 0.0;
@@ -947,7 +959,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                                   w.wid;
                     if (k + i <= a.cap) {
                         if (k + i == a.cap) store_cells(a.phi);
-                        w.template update<true>(phi, pending, wsum, a.err);
+                        w.template update<true>(phi, pending, wsum, a);
                     } else if (k + i - 1 == a.cap) {
                         // past the cap only its sum is left to do
                         float s = pending;
@@ -965,7 +977,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             dec = sh.code;
             estar = sh.estar;
             first += (uint32_t)(k / 4 - 1);
-            w.drain(a.err);
+            w.drain(a);
             base = kstar >= last ? last : before;
             from = base == 0 ? a.phi0 : base == last ? a.ck[cb] : a.ck[cb ^ 1];
         }
@@ -983,14 +995,14 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             }
             for (int j = base; j < kstar; ++j) {
                 if (WIDE && j > base && j % kResGhost == 0) {
-                    w.drain(a.err);
+                    w.drain(a);
                     refresh();
                 }
-                w.template update<false>(phi, pending, nullptr, a.err);
+                w.template update<false>(phi, pending, nullptr, a);
                 sync_sweepers();
             }
             store_cells(a.phi);
-            w.drain(a.err);
+            w.drain(a);
         }
         if (threadIdx.x == 0 && rank == 0) {
             GridState* gs = a.gs + b;
@@ -1009,19 +1021,22 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         if (a.groups >= a.B) break;
         if (threadIdx.x == 0) {
             uint4* nb = &a.box->next[group][seq & 1u];
-            if (a.fixed) {
+            if (sh.lost) {  // the others need not wait for this CTA
+                sh.grid = a.B;
+                if (!a.fixed && rank == 0 && n > 1) st_box(nb, (uint32_t)a.B, 0u, seq);
+            } else if (a.fixed) {
                 sh.grid = b + a.groups;
             } else if (rank == 0) {
                 sh.grid = a.groups + (int)atomicAdd(&a.box->queue, 1u);
                 if (n > 1) st_box(nb, (uint32_t)sh.grid, 0u, seq);
             } else {
                 uint4 v;
-                int left = kResPolls;
+                int left = a.polls;
                 do {
                     v = ld_box(nb);
                 } while (v.y != seq && --left > 0);
-                if (left <= 0) {
-                    *a.err = 1;
+                if (v.y != seq) {
+                    give_up(a, sh.lost);
                     v.x = (uint32_t)a.B;
                 }
                 sh.grid = (int)v.x;
