@@ -130,7 +130,8 @@ void hp_ctx_destroy(hp_ctx *ctx);
  * synchronises the device and returns HP_ERR_GUARD if a kernel wrote into a
  * guard zone (past the end of a workspace), HP_ERR_CUDA on a pending CUDA
  * error, HP_ERR_TIMEOUT if a bounded wait of the sweep kernel gave up since
- * the last check (its results are then void), else HP_OK. */
+ * the last check, else HP_OK.  The outputs of such a call are marked: -1
+ * sweeps, not converged, and NaN in every field. */
 hp_status hp_ctx_check(hp_ctx *ctx);
 
 /* Polls after which a wait of the grid-resident sweeps gives up, for calls

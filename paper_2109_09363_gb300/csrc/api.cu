@@ -190,7 +190,7 @@ hp_status hp_ctx_create(hp_ctx** out, hp_shape mx, int device)
         (rc = dalloc((uint8_t**)&c->box, resident_box_bytes(), &c->guards)) != HP_OK ||
         (mx.nx > 512 &&
          (rc = dalloc((uint8_t**)&c->cols, resident_columns_bytes(), &c->guards)) != HP_OK) ||
-        (rc = dalloc(&c->wait_err, 1, &c->guards)) != HP_OK) {
+        (rc = dalloc(&c->wait_err, 2, &c->guards)) != HP_OK) {
         hp_ctx_destroy(c);
         return rc;
     }

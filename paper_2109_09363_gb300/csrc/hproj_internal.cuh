@@ -122,7 +122,8 @@ struct hp_ctx {
     float* ckpt;         // [max_cells] checkpoint buffer of the resident sweep kernel
     void* box;           // exchange area of the resident sweep kernel (ResBox)
     void* cols;          // that of copied columns (ResColumns), null for max nx <= 512
-    int32_t* wait_err;   // set by a bounded wait of that kernel that gave up
+    int32_t* wait_err;   // [2] set by a bounded wait of that kernel that gave up:
+                         // since the last check, in the latest launch
     int32_t wait_limit;  // polls of its waits, 0: the compiled limits
     uint32_t epoch;      // its launches
     int32_t* host_flag;  // pinned

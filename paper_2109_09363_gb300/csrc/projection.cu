@@ -1175,12 +1175,46 @@ static int norms_kernel(const float* u, const float* v, const uint8_t* flags,
 // of the grid's partial sums (lane order, FP64) and takes their max, then
 // thread 0 the warps' results in order; a fixed order, so E_1 is the same on
 // every call.
+//
+// A grid of a launch in which a wait gave up (*lost) has no result: its outputs
+// become -1 sweeps, not converged, and NaN.
 constexpr int kFinishWarps = 8;
+
+struct Outputs {
+    const int32_t* lost;  // null: such a launch has no waits
+    float *u, *v, *p, *phi;
+    double* hist;
+    int hist_len, ny, nx;
+};
+
+__device__ void fill_nan(float* q, size_t n, int b)
+{
+    if (q)
+        for (size_t i = threadIdx.x; i < n; i += blockDim.x) q[b * n + i] = NAN;
+}
 
 __global__ void norms_finish_kernel(const float2* __restrict__ partial, int nblk, double* e1,
                                     double* einf, const GridState* gs, int32_t* iters,
-                                    uint8_t* conv, int B, double inv_cells)
+                                    uint8_t* conv, bool fixed, double inv_cells, Outputs out)
 {
+    if (out.lost && *out.lost) {
+        const int b = blockIdx.x;
+        const size_t ny = out.ny, nx = out.nx;
+        fill_nan(out.u, ny * (nx + 1), b);
+        fill_nan(out.v, (ny + 1) * nx, b);
+        fill_nan(out.p, ny * nx, b);
+        fill_nan(out.phi, ny * nx, b);
+        if (out.hist)
+            for (int i = threadIdx.x; i < out.hist_len; i += blockDim.x)
+                out.hist[(size_t)b * out.hist_len + i] = NAN;
+        if (threadIdx.x == 0) {
+            if (e1) e1[b] = NAN;
+            if (einf) einf[b] = NAN;
+            if (iters) iters[b] = -1;
+            if (conv) conv[b] = 0;
+        }
+        return;
+    }
     __shared__ double s_w[kFinishWarps];
     __shared__ float s_m[kFinishWarps];
     const int b = blockIdx.x;
@@ -1227,7 +1261,7 @@ __global__ void norms_finish_kernel(const float2* __restrict__ partial, int nblk
         if (einf) einf[b] = (double)m;
         if (gs) {
             if (iters) iters[b] = gs[b].kstar;
-            if (conv) conv[b] = (uint8_t)gs[b].converged;
+            if (conv) conv[b] = fixed ? 1 : (uint8_t)gs[b].converged;
         }
     }
 }
@@ -1251,7 +1285,8 @@ hp_status launch_div_norms_scratch(const float* u, const float* v, const uint8_t
     hp_status rc = check_launch();
     if (rc != HP_OK) return rc;
     norms_finish_kernel<<<s.batch, kFinishWarps * 32, 0, st>>>(
-        p2, nblk, e1, einf, nullptr, nullptr, nullptr, s.batch, 1.0 / ((double)s.nx * (double)s.ny));
+        p2, nblk, e1, einf, nullptr, nullptr, nullptr, false,
+        1.0 / ((double)s.nx * (double)s.ny), Outputs{});
     return check_launch();
 }
 
@@ -1513,14 +1548,11 @@ hp_status project_impl(hp_ctx* ctx, float* u, float* v, const uint8_t* flags, hp
         if ((rc = check_launch()) != HP_OK) return rc;
     }
     norms_finish_kernel<<<s.batch, kFinishWarps * 32, 0, st>>>(
-        p2, nblk, u ? e1_out : nullptr, u ? einf_out : nullptr, ctx->gs, iters_out,
-        fixed ? nullptr : conv_out, s.batch, 1.0 / ((double)s.nx * (double)s.ny));
-    if ((rc = check_launch()) != HP_OK) return rc;
-    if (fixed && conv_out) {
-        cudaError_t e = cudaMemsetAsync(conv_out, 1, (size_t)s.batch, st);
-        if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
-    }
-    return HP_OK;
+        p2, nblk, u ? e1_out : nullptr, u ? einf_out : nullptr, ctx->gs, iters_out, conv_out,
+        fixed, 1.0 / ((double)s.nx * (double)s.ny),
+        Outputs{resident ? ctx->wait_err + 1 : nullptr, u, v, p_out, phi_copy_out, e_hist, hist_len,
+                s.ny, s.nx});
+    return check_launch();
 }
 
 }  // namespace hp

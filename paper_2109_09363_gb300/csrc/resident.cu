@@ -62,15 +62,18 @@ bool res_plan(const hp_ctx* ctx, hp_shape s, ResPlan* best)
 // Per-grid state, the exchange area of `ctas` CTAs in groups (n > 1), and, for
 // a fixed number of sweeps, which grids hold values so large that a sum of
 // residuals could overflow: those stop at the first non-finite E.
-__global__ void resident_prep_kernel(GridState* gs, ResBox* box, ResColumns* cols, int B, int ctas,
-                                     int n,
+__global__ void resident_prep_kernel(GridState* gs, ResBox* box, ResColumns* cols, int32_t* err,
+                                     int B, int ctas, int n,
                                      const float* __restrict__ div,
                                      const float* __restrict__ phi0, size_t cells, uint32_t epoch,
                                      int scan)
 {
     const size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t step = (size_t)gridDim.x * blockDim.x;
-    if (id == 0) box->queue = 0u;
+    if (id == 0) {
+        box->queue = 0u;
+        err[1] = 0;
+    }
     for (size_t b = id; b < (size_t)B; b += step) gs[b].active = 1;
     if (n > 1) {
         const uint4 z = make_uint4(0, 0, 0, 0);
@@ -156,7 +159,7 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     const size_t work = a.fixed ? cells * s.batch / 8 : p.n > 1 ? (size_t)ctas * 1024 : s.batch;
     const size_t want = work / 256 + 1, most = 8 * (size_t)ctx->num_sms;
     resident_prep_kernel<<<(unsigned)(want < most ? want : most), 256, 0, st>>>(
-        ctx->gs, a.box, a.cols, s.batch, ctas, p.n, ctx->div, phi0, cells, a.epoch, a.fixed);
+        ctx->gs, a.box, a.cols, a.err, s.batch, ctas, p.n, ctx->div, phi0, cells, a.epoch, a.fixed);
     hp_status rc = check_launch();
     if (rc != HP_OK) return rc;
     cudaLaunchConfig_t cfg = {};

@@ -108,7 +108,7 @@ struct ResArgs {
     GridState* gs;
     ResBox* box;
     ResColumns* cols;   // null unless ntx > 1
-    int32_t* err;       // set to 1 when a wait gave up
+    int32_t* err;       // both set to 1 when a wait gave up
     int32_t polls, looks;  // limits of the waits (kResPolls, kResLooks)
     double* e_hist;     // [B][hist_len] or null
     int32_t hist_len;
@@ -242,7 +242,7 @@ __device__ __forceinline__ Pair pair_tree(Pair v)
 // A wait of this CTA ran out.
 __device__ __forceinline__ void give_up(const ResArgs& a, volatile int& lost)
 {
-    *a.err = 1;
+    a.err[0] = a.err[1] = 1;
     lost = 1;
 }
 

@@ -1,6 +1,7 @@
 """Bounded waits of the grid-resident sweeps made to run out (one poll each:
 no message between SMs, and no sum of several sweeps, arrives within it): the
-kernel returns, hp_ctx_check reports it, and the next call is right again.
+kernel returns, hp_ctx_check reports it, the outputs are marked (-1 sweeps, not
+converged, NaN in every field), and the next call is right again.
 Strips with one and with several columns, grids of one CTA, more grids than
 fit at once, a fixed count and a stop with a replay."""
 import pytest
@@ -16,7 +17,7 @@ SHAPES = [(1, 512, 512), (40, 300, 256), (200, 64, 128), (2, 300, 600), (12, 200
 
 def project(ctx, u, v, fl, **kw):
     a, b = u.clone(), v.clone()
-    o = hp.hp_project(ctx, a, b, fl, hp.ProjectParams(**kw))
+    o = hp.hp_project(ctx, a, b, fl, hp.ProjectParams(**kw), hist_len=kw.get("max_iters", 0))
     torch.cuda.synchronize()
     return dict(o, u=a, v=b)
 
@@ -32,12 +33,21 @@ def test_waits_that_run_out_return_and_are_reported(dev, shape, kw):  # noqa: F8
     waits = "threshold" in kw or shape != (200, 64, 128)
     ctx.set_wait_limit(1)
     for _ in range(3):
-        project(ctx, u, v, fl, **kw)
+        void = project(ctx, u, v, fl, **kw)
         if waits:
+            assert (void["iters"] == -1).all() and (void["converged"] == 0).all()
+            for k in set(ref) - {"iters", "converged"}:
+                assert torch.isnan(void[k]).all(), k
             with pytest.raises(hp.HprojError, match="status 7"):
                 ctx.check()
     ctx.set_wait_limit(0)
     got = project(ctx, u, v, fl, **kw)
     ctx.check()
     for k in ref:
-        assert torch.equal(ref[k], got[k]), k
+        assert torch.equal(torch.nan_to_num(ref[k]), torch.nan_to_num(got[k])), k
+    # outputs that carry no counts: the sweeps by themselves
+    div = torch.randn(shape, generator=torch.Generator().manual_seed(3)).to(dev)
+    phi = torch.zeros(shape, device=dev)
+    ctx.set_wait_limit(1)
+    if shape != (200, 64, 128):
+        assert torch.isnan(hp.hp_jacobi_sweeps(ctx, phi, div, fl, 41)).all()
