@@ -220,6 +220,7 @@ struct Pair {
 __device__ __forceinline__ Pair pair_add(Pair a, Pair b)
 {
     const float s = __fadd_rn(a.h, b.h);
+    if (!(fabsf(s) <= 3.402823466e38f)) return {s, 0.0f};  // the error of an infinite sum is NaN
     const float t = __fsub_rn(s, a.h);
     const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
     const float f = __fadd_rn(e, __fadd_rn(a.l, b.l));
