@@ -29,10 +29,13 @@
 // anew every 8 sweeps (through the L2 as well), which costs two exposed round
 // trips in 8 sweeps instead of one more exchange in each.
 //
-// E_k: FP32 |r| per thread and warp, then sums of float pairs (TwoSum, 48
-// bits; an FP64 addition of a warp occupies its scheduler's FP64 unit for 64
-// cycles here, and four dependent ones per round cost 0.6 us a sweep) per CTA
-// (16 warp sums) and per group (CTA partials in rank order), in rounds of four
+// E_k: FP32 |r| per thread and group of eight lanes (1,024 cells at most; over
+// whole warps the mean error against FP64 was up to 1.6 times that of FP64 sums
+// of 1,024 cells each, at 2048^2, and is now 0.5 to 1.1 times it), then sums of
+// float pairs (TwoSum, 48 bits; an FP64 addition of a warp occupies its
+// scheduler's FP64 unit for 64 cycles here, and four dependent ones per round
+// cost 0.6 us a sweep) per CTA (32 sums) and per group (CTA partials in rank
+// order), in rounds of four
 // sweeps.  Round q holds sweeps 4q..4q+3; one warp of every CTA posts the CTA
 // partials, rank 0 adds them one round later and posts the stop decision,
 // every CTA reads it one round after that, so all CTAs of a group leave the
@@ -64,6 +67,7 @@ static_assert(kResSweepers * kResRegsSweep + 128 * kResRegsHelp <= kResThreads *
 constexpr int kResLag = 3;
 constexpr int kResRing = 4;        // > kResLag: rounds between the sweeps and the decision
 constexpr int kWsumRing = 4 * kResRing;  // warp sums, by sweep
+constexpr int kResSums = 4;        // of one warp: each over eight lanes
 // A wait gives up after so many polls: of a word in the L2 (a round trip, half
 // a microsecond, so about a second) or of a barrier (suspended for a microsecond
 // at most); of a word in shared memory, which waits for a warp that waits for
@@ -71,8 +75,8 @@ constexpr int kWsumRing = 4 * kResRing;  // warp sums, by sweep
 // each for the rest of its grid (whose result is void) and takes no other grid.
 constexpr int kResPolls = 1 << 21, kResLooks = 1 << 27;
 // the sums of pairs are scaled (exactly) so that no sum of finite warp sums overflows
-constexpr float kSumScale = 1.0f / 4096.0f;
-static_assert(kResMaxCtas * kResWarps <= 4096, "warp sums of one grid");
+constexpr float kSumScale = 1.0f / 8192.0f;
+static_assert(kResMaxCtas * kResWarps * kResSums <= 8192, "FP32 sums of one grid");
 
 // Exchange area in global memory (one per context, cleared before every
 // launch): messages between neighbouring CTAs, E partials, decisions, queue.
@@ -140,9 +144,9 @@ struct ResLayout {
     static constexpr int kHalo = kCol + 2 * kColPar;
     static constexpr int kHaloPar = WX * kRowSlot;
     static constexpr int kLut = kHalo + 4 * kHaloPar;                    // [5] float2
-    static constexpr int kWsum = kLut + 64;                              // [16][8] float
+    static constexpr int kWsum = kLut + 64;                              // [16][8][4] float
     // copied columns in transit: [warp][2 sides][R][8] float
-    static constexpr int kGhost = kWsum + kWsumRing * kResWarps * 4;
+    static constexpr int kGhost = kWsum + kWsumRing * kResWarps * kResSums * 4;
     static constexpr int kBytes = kGhost + kResWarps * 2 * R * kResGhost * 4;
     static_assert(R % 4 == 0 && C % 4 == 0, "rows and columns go out four values at a time");
     static_assert(kBytes <= 227 * 1024 - 64, "shared memory of one CTA");
@@ -333,8 +337,8 @@ struct ResWarp {
 
     // phi_{k+1} from phi_k and the boundary values of message t; sends message
     // t + 1.  WITH_E: `pending` (this thread's FP32 sum of |r(phi_{k-1})|) is
-    // summed over the warp while the rows are computed, stored in *wsum by lane
-    // 0, and becomes the sum of |r(phi_k)|.
+    // summed over groups of eight lanes while the rows are computed, stored in
+    // *wsum by lanes 0..3, and becomes the sum of |r(phi_k)|.
     template <bool WITH_E>
     __device__ __forceinline__ void update(float (&phi)[R][C], float& pending, float* wsum,
                                            const ResArgs& a)
@@ -354,7 +358,10 @@ struct ResWarp {
         for (int q = 0; q < C; ++q) dsp[q] = __fsub_rn(phi[0][q], dsp[q]);
         const int s_div = L::kDiv + (wid * R * V * 32 + lane) * 16;
         const int s_code = L::kCode + (wid * R * 32 + lane) * 4;
+        // |r| in four chains, by column; with 16 rows a thread they would be 32
+        // values long, so every four rows are added up by themselves
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float sum[2] = {0.0f, 0.0f};
         float s = pending;
         // one row: differences of phi_k (each formed once: south of row r is
         // minus north of row r + 1, east of a cell minus west of the next),
@@ -425,8 +432,8 @@ struct ResWarp {
             };
             if (WITH_E) {
 #pragma unroll
-                for (int i = 0; i < 5; ++i) {  // five levels over the groups there are
-                    if (i * (R / 4) / 5 == g)
+                for (int i = 0; i < 3; ++i) {  // three levels over the groups there are
+                    if (i * (R / 4) / 3 == g)
                         s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 16 >> i));
                 }
             }
@@ -449,6 +456,11 @@ struct ResWarp {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) after(i);
             }
+            if (WITH_E && R == 16) {
+                sum[g / 2] = __fadd_rn(sum[g / 2], __fadd_rn(__fadd_rn(acc[0], acc[1]),
+                                                             __fadd_rn(acc[2], acc[3])));
+                acc[0] = acc[1] = acc[2] = acc[3] = 0.0f;
+            }
             if (WX > 1) {
                 const bool q = lane == 31;
                 // predicated, not branched around
@@ -466,9 +478,10 @@ struct ResWarp {
         }
         ++t;
         if (WITH_E) {
-            if (lane == 0) *wsum = s;
-            pending = mute ? 0.0f
-                          : __fadd_rn(__fadd_rn(acc[0], acc[1]), __fadd_rn(acc[2], acc[3]));
+            if (lane < kResSums) *wsum = s;
+            pending = mute ? 0.0f : __fadd_rn(
+                R == 16 ? sum[0] : __fadd_rn(acc[0], acc[1]),
+                R == 16 ? sum[1] : __fadd_rn(acc[2], acc[3]));
         }
     }
     template <bool P>
@@ -549,8 +562,11 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
         // (lanes look at a barrier and at words one by one: every decision
         // about a wait is taken by the warp)
         bool there = __all_sync(0xffffffffu, bar_wait(&sh.sums[slot], e / kResRing & 1u, a.polls));
-        const float* ws = s_wsum + (e * 4 + gi) % kWsumRing * kResWarps;
-        Pair sum = pair_tree({ws[li] * kSumScale, 0.0f});
+        const float4 ws = reinterpret_cast<const float4*>(
+            s_wsum)[(e * 4 + gi) % kWsumRing * kResWarps + li];
+        Pair sum = pair_tree(
+            pair_add(pair_add({ws.x * kSumScale, 0.0f}, {ws.y * kSumScale, 0.0f}),
+                     pair_add({ws.z * kSumScale, 0.0f}, {ws.w * kSumScale, 0.0f})));
         if (n > 1) {
             if (li == 0)
                 st_box(&a.box->part[cta][slot][gi], __float_as_uint(sum.h), __float_as_uint(sum.l),
@@ -956,8 +972,8 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                         __threadfence_block();
                         if (sh.stop == q) sh.act = 1;
                     }
-                    float* wsum = s_wsum + ((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
-                                  w.wid;
+                    float* wsum = s_wsum + (((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
+                                            w.wid) * kResSums + w.lane;
                     if (k + i <= a.cap) {
                         if (k + i == a.cap) store_cells(a.phi);
                         w.template update<true>(phi, pending, wsum, a);
@@ -965,9 +981,9 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                         // past the cap only its sum is left to do
                         float s = pending;
 #pragma unroll
-                        for (int off = 16; off > 0; off >>= 1)
+                        for (int off = 16; off >= kResSums; off >>= 1)
                             s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
-                        if (w.lane == 0) *wsum = s;
+                        if (w.lane < kResSums) *wsum = s;
                     }
                     if (i == 0 && k > 0 && w.lane == 0)
                         bar_arrive(&sh.sums[(first + k / 4 - 1) % kResRing]);
