@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         }
         if (threadIdx.x == 0) {
             for (int i = 0; i < 4; ++i) bar_init(&sh.full[i / 2][i % 2], 1);
-            for (int i = 0; i < kResRing; ++i) bar_init(&sh.sums[i], kResWarps);
+            for (int i = 0; i < kResRing; ++i) bar_init(&sh.sums[i], 1);
             sh.end = 0u;
             sh.lost = 0;
         }
@@ -972,6 +972,10 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                         __threadfence_block();
                         if (sh.stop == q) sh.act = 1;
                     }
+                    // behind the barrier that follows the last store of its sums (by
+                    // four lanes of each warp)
+                    if (i == 1 && k > 0 && threadIdx.x == 0)
+                        bar_arrive(&sh.sums[(first + k / 4 - 1) % kResRing]);
                     float* wsum = s_wsum + (((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
                                             w.wid) * kResSums + w.lane;
                     if (k + i <= a.cap) {
@@ -985,8 +989,6 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                             s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
                         if (w.lane < kResSums) *wsum = s;
                     }
-                    if (i == 0 && k > 0 && w.lane == 0)
-                        bar_arrive(&sh.sums[(first + k / 4 - 1) % kResRing]);
                     sync_sweepers();
                 }
             }
