@@ -25,21 +25,22 @@ struct ResPlan {
 int res_ctas(const hp_ctx* ctx) { return ctx->num_sms < kResMaxCtas ? ctx->num_sms : kResMaxCtas; }
 
 // The split with the least time: waves of groups x time per sweep of a strip,
-// measured (16 x 512^2, 8 x 256^2, 152 x 128^2 and, for columns, 2048^2 grids with
-// obstacles).  More
-// rows per thread make a longer sweep with less of it lost to the exchange,
-// fewer rows spread a grid over more SMs: 16 x 512^2 takes 5.0, 3.8 and 5.5 us
-// per sweep with 4, 8 and 16 rows (four, two waves and one), one 512^2 grid
-// 1.27, 1.83 and 3.2 us.
+// measured with all SMs at work and obstacles in every grid (38, 152 and 152
+// grids of 128^2; 19, 38 and 64 of 256^2; 16 of 512^2; 4 of 1024^2 and one of
+// 2048^2).  More rows per thread make a longer sweep with less of it lost to
+// the exchange, fewer rows spread a grid over more SMs: 16 x 512^2 takes 5.3,
+// 3.7 and 4.9 us per sweep with 4, 8 and 16 rows (four, two waves and one), one
+// 512^2 grid 1.43, 2.0 and 3.4 us.  64 x 256^2 in one wave of 16 rows took 4.5
+// us a sweep and all grids as long as the slowest; in two of 8 rows 3.6 us.
 bool res_plan(const hp_ctx* ctx, hp_shape s, ResPlan* best)
 {
     // wider than 512 cells: columns of 240, eight copied on each side
     const int width = s.nx <= 128 ? 128 : s.nx <= 256 ? 256 : s.nx <= 512 ? 512 : 1024;
     const int own = 256 - 2 * kResGhost;
     const int ntx = width == 1024 ? (s.nx + own - 1) / own : 1;
-    // us per sweep of a strip with E, on grids with obstacles, R = 4, 8, 16
+    // us per sweep of a strip with E, R = 4, 8, 16
     static const double us[4][3] = {
-        {0.72, 1.0, 1.78}, {1.12, 1.84, 3.3}, {1.27, 1.85, 4.4}, {0.0, 2.03, 3.82}};
+        {0.72, 1.03, 1.8}, {1.14, 1.95, 4.5}, {1.35, 1.87, 4.9}, {0.0, 1.95, 3.75}};
     const int ctas = res_ctas(ctx);
     double least = 0.0;
     bool found = false;
