@@ -35,12 +35,11 @@
 // float pairs (TwoSum, 48 bits; an FP64 addition of a warp occupies its
 // scheduler's FP64 unit for 64 cycles here, and four dependent ones per round
 // cost 0.6 us a sweep) per CTA (32 sums) and per group (CTA partials in rank
-// order), in rounds of four
-// sweeps.  Round q holds sweeps 4q..4q+3; one warp of every CTA posts the CTA
-// partials, rank 0 adds them one round later and posts the stop decision,
-// every CTA reads it one round after that, so all CTAs of a group leave the
-// loop at the same sweep and go back to the last checkpoint of phi at or below
-// k* (one every 32 sweeps), from which they replay the sweeps to k* exactly.
+// order), in rounds of four sweeps.  Round q holds sweeps 4q..4q+3; one warp of
+// every CTA posts the CTA partials, that of rank 0 adds them and posts the stop
+// decision, which every CTA reads at the same sweep (res_lag), so all CTAs of a
+// group leave the loop together and go back to the last checkpoint of phi at or below
+// k* (ckpt_step), from which they replay the sweeps to k* exactly.
 // The comparison with the threshold is made in FP64 whenever the FP32 head of
 // the sum is within 1e-6 of it.  phi at the cap is kept aside as it passes, so
 // a grid that reaches its cap replays nothing; a run of fixed length needs
@@ -63,8 +62,15 @@ constexpr int kResMaxCtas = 192;   // CTAs of one launch (one per SM)
 constexpr int kResRegs = 168, kResRegsSweep = 232, kResRegsHelp = 40;
 static_assert(kResSweepers * kResRegsSweep + 128 * kResRegsHelp <= kResThreads * kResRegs,
               "the split waits forever for registers the launch does not have");
-// a decision about sweep j is known everywhere before sweep 4 (j / 4 + kResLag)
+// A decision about sweep j is known everywhere before sweep 4 (j / 4 + lag), for
+// the lag of the loop index at which it is read.  A single CTA has it within a
+// sweep.  Between CTAs it takes up to 8 us (144 of them), more than two sweeps:
+// waiting for it costs that much in each round (2048^2: 3.6 us a sweep with a lag
+// of three, 4.5 with two), sweeping on costs four more sweeps once.  So the first
+// two rounds, where most hybrid projections stop, are waited for and the others
+// are not.
 constexpr int kResLag = 3;
+__device__ __forceinline__ int res_lag(int k, int n) { return n == 1 || k < 12 ? 2 : kResLag; }
 constexpr int kResRing = 4;        // > kResLag: rounds between the sweeps and the decision
 constexpr int kWsumRing = 4 * kResRing;  // warp sums, by sweep
 constexpr int kResSums = 4;        // of one warp: each over eight lanes
@@ -105,7 +111,7 @@ struct ResArgs {
     // from it) when these may already be storing phi_{k*}
     float* phi;
     // checkpoint buffers [B][ny][nx]; phi0 may be ck[1], which is first written
-    // at sweep 64, when every strip has read phi_0 and no replay starts from it
+    // at sweep 32, when every strip has read phi_0 and no replay starts from it
     float* ck[2];
     const float* div;   // [B][ny][nx]
     const uint8_t* mask;
@@ -191,19 +197,29 @@ __device__ __forceinline__ void bar_arrive(uint64_t* b)
                  : "memory");
 }
 
-// whether the phase of this parity has completed; bounded
-__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, int polls)
+// whether the phase of this parity has completed; a poll is suspended for a
+// microsecond at most
+__device__ __forceinline__ bool bar_try(uint64_t* b, uint32_t parity)
 {
-    uint32_t done = 0;
-    do {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(res_smem(b)), "r"(parity), "r"(1000u)  // ns
-            : "memory");
-    } while (!done && --polls > 0);
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(res_smem(b)), "r"(parity), "r"(1000u)  // ns
+        : "memory");
     return done != 0;
+}
+
+// the same, after up to `limit` polls
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, const volatile int& limit)
+{
+    bool done = bar_try(b, parity);
+    if (!done) {
+        int polls = limit;
+        while (!done && --polls > 0) done = bar_try(b, parity);
+    }
+    return done;
 }
 
 // named barriers: 1 the sweep warps, 2 these and the helper of the E rounds
@@ -244,11 +260,11 @@ __device__ __forceinline__ Pair pair_tree(Pair v)
     return v;
 }
 
-// A wait of this CTA ran out.
-__device__ __forceinline__ void give_up(const ResArgs& a, volatile int& lost)
+// A wait of this CTA ran out: the others wait for one poll only from now on.
+__device__ __forceinline__ void give_up(const ResArgs& a, volatile int& limit)
 {
     a.err[0] = a.err[1] = 1;
-    lost = 1;
+    limit = 1;
 }
 
 template <int C, int R, int WX>
@@ -269,10 +285,9 @@ struct ResWarp {
     int out_r, out_c; // of this warp's own rows and column
     int in_h;         // of the row received from the neighbouring CTA
     uint64_t* full;   // [parity]: it is there
-    volatile int* lost;  // ResShared::lost
+    volatile int* limit;  // ResShared::limit
     uint4* tx;        // [parity][word] to the neighbouring CTA, this lane
     uint32_t t;       // messages sent (= received and being waited for) so far
-    bool dead;        // a wait of this lane gave up: do not wait any more
 
     __device__ __forceinline__ void ld_row(int off, float (&v)[C]) const
     {
@@ -293,10 +308,7 @@ struct ResWarp {
     // the row of message t, from the helper that receives it; bounded
     __device__ __forceinline__ void receive(float (&v)[C], const ResArgs& a)
     {
-        if (!bar_wait(full + (t & 1u), (t - 1) >> 1 & 1u, dead ? 1 : a.polls)) {
-            dead = true;
-            give_up(a, *lost);
-        }
+        if (!bar_wait(full + (t & 1u), (t - 1) >> 1 & 1u, *limit)) give_up(a, *limit);
         ld_row(in_h + (t & 1u ? L::kHaloPar : 0), v);
     }
     __device__ __forceinline__ void send(const float (&v)[C], uint32_t tag) const
@@ -500,14 +512,20 @@ struct ResShared {
     int kstar, code;           // k*; 1 converged, 2 not
     double estar;
     int act;                   // 1: leave the sweep loop
-    volatile int lost;         // 1: a wait gave up
+    int begun;                 // rounds begun by then
+    volatile int limit;        // polls of a wait; 1 once one has given up
     int grid;                  // next grid of the group
 };
 
-// Checkpoints: the first at 32 sweeps (more than the sweeps a decision takes),
-// later ones further apart (one costs about four sweeps of its CTA; replaying
-// from one costs at most an eighth of the sweeps done)
-__device__ __forceinline__ int ckpt_step(int k) { return k < 256 ? 32 : k < 1024 ? 64 : 128; }
+// Sweeps from checkpoint k to the next.  A store of a strip costs two to four of
+// its sweeps, a stop replays half a step on average, so the step grows as the
+// root of the sweeps done; 16 sweeps or more, since a decision may take 12.
+// (With 32 from the start, a stop at sweep 20 or 60 took up to 1.4 times as
+// long: 256 x 128^2 323 and 243 us, 410 and 330 us.)
+__device__ __forceinline__ int ckpt_step(int k)
+{
+    return k < 64 ? 16 : k < 256 ? 32 : k < 1024 ? 64 : 128;
+}
 
 // Helper warp: rows from the neighbouring CTA on one side into shared memory.
 template <int C, int R, int WX>
@@ -518,11 +536,12 @@ __device__ __forceinline__ void res_receiver(const ResArgs& a, uint8_t* sm, ResS
     constexpr int W = 2 * L::V;  // words per source lane
     const int lane = threadIdx.x & 31;
     for (uint32_t t = 1;; ++t) {
+        const int limit = __shfl_sync(0xffffffffu, sh.limit, 0);  // the warp's
 #pragma unroll 1
         for (int x = 0; x < WX; ++x) {
             const uint4* p = &a.box->row[cta][side][t & 1u][32 * x + lane];
             uint4 v[W];
-            int left = a.polls;
+            int left = limit;
             for (;;) {
                 bool ok = true;
 #pragma unroll
@@ -534,7 +553,7 @@ __device__ __forceinline__ void res_receiver(const ResArgs& a, uint8_t* sm, ResS
                 const uint32_t end = sh.end;
                 if (__any_sync(0xffffffffu, end != 0 && t > end)) return;
                 if (--left <= 0) {
-                    give_up(a, sh.lost);
+                    give_up(a, sh.limit);
                     return;
                 }
             }
@@ -561,7 +580,8 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
         const uint32_t e = first + q, tag = e + 1, slot = e % kResRing;
         // (lanes look at a barrier and at words one by one: every decision
         // about a wait is taken by the warp)
-        bool there = __all_sync(0xffffffffu, bar_wait(&sh.sums[slot], e / kResRing & 1u, a.polls));
+        bool there = __all_sync(
+            0xffffffffu, bar_wait(&sh.sums[slot], e / kResRing & 1u, sh.limit));
         const float4 ws = reinterpret_cast<const float4*>(
             s_wsum)[(e * 4 + gi) % kWsumRing * kResWarps + li];
         Pair sum = pair_tree(
@@ -575,7 +595,7 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
                 sum = {0.0f, 0.0f};
                 for (int i = li; i < n; i += 32) {  // four loads in flight
                     uint4 v[4];
-                    int left = there ? a.polls : 1;
+                    int left = sh.limit;
                     bool ok;
                     do {
                         ok = true;
@@ -618,7 +638,7 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
                 st_box(&a.box->dec[group][slot], (uint32_t)code, (uint32_t)ks, tag);
         } else {
             uint4 v;
-            int left = there ? a.polls : 1;
+            int left = sh.limit;
             do {
                 v = ld_box(&a.box->dec[group][slot]);
             } while ((v.y != tag || v.w != tag) && --left > 0);
@@ -626,7 +646,7 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
             code = there ? (int)v.x : 2;
             ks = there ? (int)v.z : 0;
         }
-        if (!there) give_up(a, sh.lost);
+        if (!there) give_up(a, sh.limit);
         __syncwarp();
         if (lane == 0) {
             if (code != 0) {
@@ -649,12 +669,12 @@ __device__ __forceinline__ void res_rounds(const ResArgs& a, const float* s_wsum
 template <int R, int WX>
 __device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float (&phi)[R][8],
                                             int cta, int wid, int lane, bool left, bool right,
-                                            uint32_t m, bool& dead, volatile int& lost)
+                                            uint32_t m, volatile int& limit)
 {
     using L = ResLayout<8, R, WX>;
     constexpr int W = R / 8;  // words per lane and side
     float* stage = reinterpret_cast<float*>(sm + L::kGhost) + wid * 2 * R * kResGhost;
-    dead = __any_sync(0xffffffffu, dead);  // the polls below are the warp's
+    __syncwarp();
     if (lane == 1 || lane == 30) {
         float4* dst = reinterpret_cast<float4*>(stage + (lane == 1 ? 0 : R * kResGhost));
 #pragma unroll
@@ -681,7 +701,7 @@ __device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float
         if (side ? !right : !left) continue;
         const uint4* box = a.cols->w[cta][side][m & 1u][wid][0];
         uint4 v[W];
-        int polls = dead ? 1 : a.polls;
+        int polls = __shfl_sync(0xffffffffu, limit, 0);  // the warp's
         for (;;) {
             bool ok = true;
 #pragma unroll
@@ -691,8 +711,7 @@ __device__ __forceinline__ void res_columns(const ResArgs& a, uint8_t* sm, float
             }
             if (__all_sync(0xffffffffu, ok)) break;
             if (--polls <= 0) {
-                dead = true;
-                give_up(a, lost);
+                give_up(a, limit);
                 break;
             }
         }
@@ -749,7 +768,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             for (int i = 0; i < 4; ++i) bar_init(&sh.full[i / 2][i % 2], 1);
             for (int i = 0; i < kResRing; ++i) bar_init(&sh.sums[i], 1);
             sh.end = 0u;
-            sh.lost = 0;
+            sh.limit = a.polls;
         }
     }
     __syncthreads();
@@ -761,11 +780,10 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
             uint32_t first = 0;
             while (b < a.B) {
                 sync_grid();  // the sweep warps have set the grid up
-                if (!a.fixed || a.gs[b].wild == a.epoch) {
-                    res_rounds(a, s_wsum, sh, b, first);
-                    first += (uint32_t)(sh.stop + kResLag - 1);
-                }
+                const bool with_e = !a.fixed || a.gs[b].wild == a.epoch;
+                if (with_e) res_rounds(a, s_wsum, sh, b, first);
                 sync_grid();  // the grid is done
+                if (with_e) first += (uint32_t)sh.begun;
                 if (a.groups >= a.B) break;
                 sync_grid();
                 b = sh.grid;
@@ -795,8 +813,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         w.in_h = L::kHalo + side * 2 * L::kHaloPar + w.wx * L::kRowSlot + w.lane * 16;
     }
     w.t = 0;
-    w.dead = false;
-    w.lost = &sh.lost;
+    w.limit = &sh.limit;
     const bool left = WIDE && tx > 0, right = WIDE && tx < ntx - 1;
     const int x0 = (WIDE ? tx * (32 * C - 2 * kResGhost) - kResGhost : 0) + (w.wx * 32 + w.lane) * C;
     const int y0 = (ty * L::WY + w.wy) * R;
@@ -837,44 +854,57 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
     while (b < a.B) {
         ++seq;
         const size_t gbase = (size_t)b * ny * nx;
+        // register rows r_lo .. r_hi - 1 are rows of the grid
+        const int r_lo = w.flip ? max(0, y0 + R - ny) : 0;
+        const int r_hi = w.flip ? R : min(R, ny - y0);
+        const size_t first_cell = gbase + (size_t)row_of(0) * nx + x0;
+        const ptrdiff_t row_step = w.flip ? -(ptrdiff_t)nx : (ptrdiff_t)nx;
+        // (loads and stores of 128 cells, several times in the kernel: written
+        // for few instructions, since a call's first sweeps wait for the
+        // kernel's code to be fetched)
         auto load_cells = [&](const float* src, bool masked, bool v4) {
+            const float* line = src + first_cell;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int y = row_of(r);
+            for (int r = 0; r < R; ++r, line += row_step) {
+                const bool in = src && r >= r_lo && r < r_hi;
+                if (v4) {
 #pragma unroll
-                for (int h = 0; h < C; h += 4) {
-                    float f[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                    if (y < ny && src) {
-                        const size_t o = gbase + (size_t)y * nx;
-                        load_row4(src + o, x0 + h, nx, v4, f);
-                        if (masked) {
-                            const uint32_t m4 = load_mask4(a.mask + o, x0 + h, nx, vec);
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                if (((m4 >> (8 * q)) & 15u) == 0u) f[q] = 0.0f;
-                        }
+                    for (int h = 0; h < C; h += 4) {
+                        float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        if (in && x0 + h >= 0 && x0 + h < nx)
+                            f = *reinterpret_cast<const float4*>(line + h);
+                        phi[r][h] = f.x; phi[r][h + 1] = f.y;
+                        phi[r][h + 2] = f.z; phi[r][h + 3] = f.w;
                     }
+                } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) phi[r][h + q] = f[q];
+                    for (int q = 0; q < C; ++q)
+                        phi[r][q] = in && x0 + q >= 0 && x0 + q < nx ? line[q] : 0.0f;
+                }
+                if (masked) {
+                    const uint32_t code =
+                        reinterpret_cast<const uint32_t*>(sm + L::kCode)[(w.wid * R + r) * 32 + w.lane];
+#pragma unroll
+                    for (int q = 0; q < C; ++q)
+                        if (!((code >> (4 * q)) & 15u)) phi[r][q] = 0.0f;
                 }
             }
         };
         auto store_cells = [&](float* dst) {
+            float* line = dst + first_cell;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int y = row_of(r);
-                if (y >= ny || copy) continue;
-                float* line = dst + gbase + (size_t)y * nx;
+            for (int r = 0; r < R; ++r, line += row_step) {
+                const bool in = !copy && r >= r_lo && r < r_hi;
+                if (vec) {
 #pragma unroll
-                for (int h = 0; h < C; h += 4) {
-                    if (vec && x0 + h + 3 < nx) {
-                        *reinterpret_cast<float4*>(line + x0 + h) = make_float4(
-                            phi[r][h], phi[r][h + 1], phi[r][h + 2], phi[r][h + 3]);
-                    } else {
+                    for (int h = 0; h < C; h += 4)
+                        if (in && x0 + h < nx)
+                            *reinterpret_cast<float4*>(line + h) = make_float4(
+                                phi[r][h], phi[r][h + 1], phi[r][h + 2], phi[r][h + 3]);
+                } else {
 #pragma unroll
-                        for (int q = h; q < h + 4; ++q)
-                            if (x0 + q < nx) line[x0 + q] = phi[r][q];
-                    }
+                    for (int q = 0; q < C; ++q)
+                        if (in && x0 + q < nx) line[q] = phi[r][q];
                 }
             }
         };
@@ -883,8 +913,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         auto refresh = [&]() {
             if constexpr (WIDE) {
                 ++fetched;
-                res_columns<R, WX>(a, sm, phi, cta, w.wid, w.lane, left, right, fetched, w.dead,
-                                   sh.lost);
+                res_columns<R, WX>(a, sm, phi, cta, w.wid, w.lane, left, right, fetched, sh.limit);
                 w.publish(phi);
                 sync_sweepers();
             }
@@ -935,53 +964,95 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         sync_grid();
 
         const bool with_e = !a.fixed || a.gs[b].wild == a.epoch;
-        int base = 0;  // the iterate that a replay would start from
-        const float* from = a.phi0;
-        if (with_e) {
+        if (!with_e) {
+            for (int j = 0; j < kstar; ++j) {
+                if (WIDE && j > 0 && j % kResGhost == 0) {
+                    w.drain(a);
+                    refresh();
+                }
+                w.template update<false>(phi, pending, nullptr, a);
+                sync_sweepers();
+            }
+            store_cells(a.phi);
+            w.drain(a);
+        } else {
+            // Four sweeps at a time; round q needs the sums of sweeps 4q .. 4q+3,
+            // the last stored during sweep 4q + 4.  A replay from phi_0 or the
+            // checkpoint at or below k* to phi_{k*} takes the same loop (and
+            // leaves its sums unread): the code of another one, 94 KB with 16
+            // rows, would have to be fetched first, which took as long as five
+            // sweeps (4 x 1024^2, stop at sweep 3: 250 and 200 us).
             int last = 0, before = 0, cb = 1;  // latest checkpoints, buffer of the latest
-            // four sweeps at a time; round q needs the sums of sweeps 4q .. 4q+3,
-            // the last stored during sweep 4q + 4
-            int k = 0;
-            for (;; k += 4) {
-                if (sh.act != 0) break;
-                if (k == last + ckpt_step(last) && k <= a.cap) {
+            bool replay = false;
+            for (int k = 0;; k += 4) {
+                bool loaded = false;
+                if (!replay && sh.act != 0) {
+                    kstar = sh.kstar;
+                    dec = sh.code;
+                    estar = sh.estar;
+                    first += (uint32_t)(k / 4 - 1);
+                    w.drain(a);
+                    if (kstar == a.cap) break;  // phi has been stored
+                    const int base = kstar >= last ? last : before;
+                    load_cells(base == 0 ? a.phi0 : a.ck[base == last ? cb : cb ^ 1], base == 0,
+                               vec && (base != 0 || a.phi0_vec));
+                    k = base;
+                    replay = loaded = true;
+                    sync_sweepers();
+                    if (!WIDE || base == 0) {
+                        w.publish(phi);
+                        sync_sweepers();
+                    }
+                }
+                // of the four: sweeps to do, and phi to be kept before one of them
+                const int todo = (replay ? kstar : a.cap + 1) - k;
+                int keep_at = replay ? todo : todo - 1;
+                float* keep = a.phi;
+                if (keep_at > 3 && !replay && k == last + ckpt_step(last)) {
                     cb ^= 1;
-                    store_cells(a.ck[cb]);
+                    keep = a.ck[cb];
+                    keep_at = 0;
                     before = last;
                     last = k;
                 }
-                if (WIDE && k > 0 && k % kResGhost == 0 && k <= a.cap) {
-                    w.drain(a);
+                const bool one_thread = threadIdx.x == kResSweepers / 2 && !replay;
+                if (WIDE && k > 0 && k % kResGhost == 0 && (todo > 0 || loaded)) {
+                    if (!loaded) w.drain(a);
                     refresh();
                 }
 #pragma unroll 1
                 for (int i = 0; i < 4; ++i) {
-                    if (i == 2 && threadIdx.x == 0 && k + 4 >= 4 * kResLag) {
-                        // the decision of round k / 4 + 1 - kResLag: long there
-                        const int q = k / 4 + 1 - kResLag;
-                        int left = a.looks;
+                    // (behind the barrier that follows the last store of its sums)
+                    if (i == 1 && one_thread && k > 0)
+                        bar_arrive(&sh.sums[(first + k / 4 - 1) % kResRing]);
+                    const int lag = res_lag(k, n);
+                    if (i == 3 && one_thread && k + 4 >= 4 * lag) {
+                        // the decision of round k / 4 + 1 - lag: mostly there
+                        const int q = k / 4 + 1 - lag;
+                        int left = sh.limit == 1 ? 1 : a.looks;
                         while (sh.rounds <= q && --left > 0) {
                         }
                         if (sh.rounds <= q) {
-                            give_up(a, sh.lost);
+                            give_up(a, sh.limit);
                             sh.kstar = 0;
                             sh.code = 2;
                             sh.estar = 0.0;
                             sh.stop = q;
                         }
                         __threadfence_block();
-                        if (sh.stop == q) sh.act = 1;
+                        if (sh.stop == q) {
+                            sh.begun = k / 4;
+                            sh.act = 1;
+                        }
                     }
-                    // behind the barrier that follows the last store of its sums (by
-                    // four lanes of each warp)
-                    if (i == 1 && k > 0 && threadIdx.x == 0)
-                        bar_arrive(&sh.sums[(first + k / 4 - 1) % kResRing]);
                     float* wsum = s_wsum + (((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
                                             w.wid) * kResSums + w.lane;
-                    if (k + i <= a.cap) {
-                        if (k + i == a.cap) store_cells(a.phi);
+                    if (i == keep_at) store_cells(keep);
+                    if (i < todo) {
                         w.template update<true>(phi, pending, wsum, a);
-                    } else if (k + i - 1 == a.cap) {
+                    } else if (replay) {
+                        break;
+                    } else if (i == todo) {
                         // past the cap only its sum is left to do
                         float s = pending;
 #pragma unroll
@@ -991,37 +1062,11 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     }
                     sync_sweepers();
                 }
-            }
-            kstar = sh.kstar;
-            dec = sh.code;
-            estar = sh.estar;
-            first += (uint32_t)(k / 4 - 1);
-            w.drain(a);
-            base = kstar >= last ? last : before;
-            from = base == 0 ? a.phi0 : base == last ? a.ck[cb] : a.ck[cb ^ 1];
-        }
-        if (!with_e || kstar != a.cap) {
-            // ---- from phi_0 or the checkpoint at or below k* to phi_{k*}
-            if (with_e) {
-                load_cells(from, base == 0, vec && (base != 0 || a.phi0_vec));
-                sync_sweepers();
-                if (WIDE && base > 0) {
-                    refresh();
-                } else {
-                    w.publish(phi);
-                    sync_sweepers();
-                }
-            }
-            for (int j = base; j < kstar; ++j) {
-                if (WIDE && j > base && j % kResGhost == 0) {
+                if (replay && kstar < k + 4) {
                     w.drain(a);
-                    refresh();
+                    break;
                 }
-                w.template update<false>(phi, pending, nullptr, a);
-                sync_sweepers();
             }
-            store_cells(a.phi);
-            w.drain(a);
         }
         if (threadIdx.x == 0 && rank == 0) {
             GridState* gs = a.gs + b;
@@ -1040,7 +1085,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         if (a.groups >= a.B) break;
         if (threadIdx.x == 0) {
             uint4* nb = &a.box->next[group][seq & 1u];
-            if (sh.lost) {  // the others need not wait for this CTA
+            if (sh.limit == 1) {  // a wait gave up: the others need not wait for this CTA
                 sh.grid = a.B;
                 if (!a.fixed && rank == 0 && n > 1) st_box(nb, (uint32_t)a.B, 0u, seq);
             } else if (a.fixed) {
@@ -1050,12 +1095,12 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                 if (n > 1) st_box(nb, (uint32_t)sh.grid, 0u, seq);
             } else {
                 uint4 v;
-                int left = a.polls;
+                int left = sh.limit;
                 do {
                     v = ld_box(nb);
                 } while (v.y != seq && --left > 0);
                 if (v.y != seq) {
-                    give_up(a, sh.lost);
+                    give_up(a, sh.limit);
                     v.x = (uint32_t)a.B;
                 }
                 sh.grid = (int)v.x;
