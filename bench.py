@@ -1209,7 +1209,7 @@ def main():
                            sweep_kernel=args.sweep_kernel)
     # the grid-resident kernel runs when the library picks it (0) or it is
     # asked for (4) and the SMs hold a grid of this shape
-    resident = args.sweep_kernel in (0, 4) and hp.hp_resident_clusters(ctx, B, N, N) > 0
+    resident = args.sweep_kernel in (0, 4) and hp.hp_resident_grids(ctx, B, N, N) > 0
     streaming = not resident and streaming_chosen(args.sweep_kernel, B * N * N)
     per_launch = 1 if streaming else T_BLOCK
     stream = torch.cuda.current_stream()
@@ -1309,7 +1309,7 @@ def main():
                     "peak": alu_peak, "unit": "TOP/s", "frac": alu_achieved / alu_peak,
                     "traffic": traffic, "peak_kind": "derived: SMs x 128 FP32 lanes x max clock",
                     "ops_per_cell_update": OPS_PER_CELL_UPDATE, "sweep_ms_batch": t_sweep_ms,
-                    "clusters_resident": hp.hp_resident_clusters(ctx, B, N, N),
+                    "grids_resident": hp.hp_resident_grids(ctx, B, N, N),
                     "hbm_effective": {"achieved": hbm_eff, "peak": peak, "unit": "GB/s",
                                       "frac": hbm_eff / peak, "peak_kind": peak_kind,
                                       "note": "13 B per cell-sweep of a sweep that streams "

@@ -203,12 +203,16 @@ hp_status hp_jacobi_sweeps(hp_ctx *ctx, const float *phi_in, const float *div,
 hp_status hp_jacobi_target(hp_ctx *ctx, const float *div, const uint8_t *flags, int32_t n,
                            float *target_out, hp_shape shape, void *stream);
 
-/* Number of grids of this shape that the grid-resident sweep kernel
- * (sweep_kernel = 4) holds on the device at once, each cut into strips of
- * whole rows on one SM each (their height by the batch: the fewer grids, the
- * more SMs per grid); 0 for grids above 512 x 512 cells (128 x 128 tiles
- * beyond 16).  Host query only (no kernel launch); 0 for a NULL context or an
+/* Number of grids of this shape that a launch of the grid-resident sweep
+ * kernel (sweep_kernel = 0 or 4) holds on the device at once, each cut into
+ * strips of one SM (their height by the batch: the fewer grids, the more SMs
+ * per grid); 0 for shapes that hp_project gives to the temporally blocked
+ * kernel.  Host query only (no kernel launch); 0 for a NULL context or an
  * invalid shape. */
+int32_t hp_resident_grids(hp_ctx *ctx, hp_shape shape);
+
+/* The same for grids of up to 16 tiles of 128 x 128 cells (512 x 512), and 0
+ * for larger ones whichever kernel serves them. */
 int32_t hp_resident_clusters(hp_ctx *ctx, hp_shape shape);
 
 /* Parameters of the plume driver step (Sec. 2.2: semi-Lagrangian advection

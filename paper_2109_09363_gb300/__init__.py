@@ -64,6 +64,7 @@ _SIGS = {
     "hp_jacobi_sweeps": (ctypes.c_int, [_P, _P, _P, _P, _P, ctypes.c_int32, _P, hp_shape, _P]),
     "hp_jacobi_target": (ctypes.c_int, [_P, _P, _P, ctypes.c_int32, _P, hp_shape, _P]),
     "hp_div_norms_noalloc": (ctypes.c_int, [_P, _P, _P, _P, _P, hp_shape, _P]),
+    "hp_resident_grids": (ctypes.c_int32, [_P, hp_shape]),
     "hp_resident_clusters": (ctypes.c_int32, [_P, hp_shape]),
     "hp_advect_step": (ctypes.c_int, [_P, _P, _P, _P, _P, _P, _P, hp_shape,
                                       ctypes.POINTER(hp_plume_params), _P]),
@@ -246,10 +247,16 @@ def hp_divergence(u, v, flags, div_out=None, stream=None):
     return div_out
 
 
+def hp_resident_grids(ctx: Context, batch: int, ny: int, nx: int) -> int:
+    """Grids of this shape that a launch of the grid-resident sweep kernel
+    (sweep_kernel 0 or 4) holds at once; 0 for shapes that hp_project gives to
+    the temporally blocked kernel."""
+    return int(load_library().hp_resident_grids(ctx.handle, hp_shape(batch, ny, nx)))
+
+
 def hp_resident_clusters(ctx: Context, batch: int, ny: int, nx: int) -> int:
-    """Grids of this shape the grid-resident sweep kernel (sweep_kernel = 4)
-    holds at once; 0 when it cannot run the shape (hp_project then uses the
-    temporally blocked kernel)."""
+    """hp_resident_grids for grids of up to 16 tiles of 128 x 128 cells; 0 for
+    larger ones, whichever kernel serves them."""
     return int(load_library().hp_resident_clusters(ctx.handle, hp_shape(batch, ny, nx)))
 
 

@@ -104,13 +104,11 @@ __global__ void resident_prep_kernel(GridState* gs, ResBox* box, ResColumns* col
 size_t resident_box_bytes() { return sizeof(ResBox); }
 size_t resident_columns_bytes() { return sizeof(ResColumns); }
 
-// Grids of shape s held on chip at once; 0 above 512 x 512 cells.
+// Grids of shape s held on chip at once by a launch; 0 when none is made.
 int resident_capacity(hp_ctx* ctx, hp_shape s)
 {
-    const int tiles = ((s.nx + 127) / 128) * ((s.ny + 127) / 128);
     ResPlan p;
-    if (tiles > 16 || !res_plan(ctx, s, &p)) return 0;
-    return res_ctas(ctx) / p.n;
+    return res_plan(ctx, s, &p) ? res_ctas(ctx) / p.n : 0;
 }
 
 hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bool fixed,
@@ -182,8 +180,18 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
 
 }  // namespace hp
 
-extern "C" int32_t hp_resident_clusters(hp_ctx* ctx, hp_shape s)
+extern "C" {
+
+int32_t hp_resident_grids(hp_ctx* ctx, hp_shape s)
+{
+    return ctx && hp::shape_ok(s) ? hp::resident_capacity(ctx, s) : 0;
+}
+
+int32_t hp_resident_clusters(hp_ctx* ctx, hp_shape s)
 {
     if (!ctx || !hp::shape_ok(s)) return 0;
-    return hp::resident_capacity(ctx, s);
+    const int tiles = ((s.nx + 127) / 128) * ((s.ny + 127) / 128);
+    return tiles > 16 ? 0 : hp::resident_capacity(ctx, s);
 }
+
+}  // extern "C"
