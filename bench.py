@@ -1114,6 +1114,29 @@ def profile_train(batch, n, norm=1, arch="multiscale") -> int:
     return 0
 
 
+def result_line(line):
+    """The result line: the headline and what qualifies it, floats of seven
+    digits, below 2 kB (readers that keep the end of stdout lost the full line,
+    26 kB with every network's arms, which goes to stderr)."""
+    keep = {"config": [k for k in line["config"] if k != "iters_per_grid"],
+            "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                         "peak_kind"),
+            "clocks": ("sm_mhz", "sm_max_mhz", "reasons"),
+            "hybrid_vs_plain": ("best_network_equal_threshold",),
+            "cpu_baseline": ("value", "unit", "cores", "kind", "sample")}
+    drop = ("hybrid", "paper_times", "pdnn_training", "driver_step", "stencil_roofline")
+
+    def short(o):
+        if isinstance(o, float):
+            return float(f"{o:.7g}")
+        if isinstance(o, dict):
+            return {k: short(v) for k, v in o.items()}
+        return [short(v) for v in o] if isinstance(o, (list, tuple)) else o
+
+    return short({k: {q: v[q] for q in keep[k] if q in v} if k in keep else v
+                  for k, v in line.items() if k not in drop})
+
+
 def main():
     global T_BLOCK
     ap = argparse.ArgumentParser()
@@ -1462,7 +1485,8 @@ def main():
         line["stencil_roofline"] = stencil
         if ws == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_oracle_sample(u_np, v_np, fl_np, gpu=gpu_result)
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"details": line}), file=sys.stderr, flush=True)
+        print(json.dumps(result_line(line)), flush=True)
     ctx.close()
     if ws > 1:
         dist.destroy_process_group()
