@@ -215,6 +215,11 @@ int32_t hp_resident_grids(hp_ctx *ctx, hp_shape shape);
  * for larger ones whichever kernel serves them. */
 int32_t hp_resident_clusters(hp_ctx *ctx, hp_shape shape);
 
+/* SMs that the grid-resident sweeps of this context may take, for calls from
+ * now on (0 = all): fewer where other work is to run beside them.  Shapes that
+ * do not fit go to the temporally blocked kernel. */
+hp_status hp_ctx_set_resident_sms(hp_ctx *ctx, int32_t sms);
+
 /* Parameters of the plume driver step (Sec. 2.2: semi-Lagrangian advection
  * of the density and of the velocity, then the external force by forward
  * Euler, giving u* for the projection).

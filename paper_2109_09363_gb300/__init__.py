@@ -65,6 +65,7 @@ _SIGS = {
     "hp_jacobi_target": (ctypes.c_int, [_P, _P, _P, ctypes.c_int32, _P, hp_shape, _P]),
     "hp_div_norms_noalloc": (ctypes.c_int, [_P, _P, _P, _P, _P, hp_shape, _P]),
     "hp_resident_grids": (ctypes.c_int32, [_P, hp_shape]),
+    "hp_ctx_set_resident_sms": (ctypes.c_int, [_P, ctypes.c_int32]),
     "hp_resident_clusters": (ctypes.c_int32, [_P, hp_shape]),
     "hp_advect_step": (ctypes.c_int, [_P, _P, _P, _P, _P, _P, _P, hp_shape,
                                       ctypes.POINTER(hp_plume_params), _P]),
@@ -191,6 +192,10 @@ class Context:
         """Polls after which a wait of the grid-resident sweeps gives up (0:
         the compiled limits)."""
         _check(load_library().hp_ctx_set_wait_limit(self._h, int(polls)))
+
+    def set_resident_sms(self, sms: int):
+        """SMs that the grid-resident sweeps may take (0: all)."""
+        _check(load_library().hp_ctx_set_resident_sms(self._h, int(sms)))
 
     def close(self):
         if self._h:

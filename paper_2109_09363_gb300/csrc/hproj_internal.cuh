@@ -126,6 +126,8 @@ struct hp_ctx {
                          // since the last check, in the latest launch
     int32_t wait_limit;  // polls of its waits, 0: the compiled limits
     uint32_t epoch;      // its launches
+    int32_t res_sms;     // SMs it may take, 0: all
+    int8_t res_known[4][3];  // its instances (width, rows): 1 run here, -1 do not, 0 not looked up
     int32_t* host_flag;  // pinned
     // cached conditional-graph loop
     cudaGraphExec_t graph_exec;

@@ -20,9 +20,36 @@ struct ResPlan {
     int width, R, n, ntx, groups;
 };
 
+int width_class(int width) { return width == 128 ? 0 : width == 256 ? 1 : width == 512 ? 2 : 3; }
+
 // CTAs of a cooperative launch that fit on the device: one per SM (every
 // instance needs most of an SM's registers)
-int res_ctas(const hp_ctx* ctx) { return ctx->num_sms < kResMaxCtas ? ctx->num_sms : kResMaxCtas; }
+int res_ctas(const hp_ctx* ctx)
+{
+    const int ctas = ctx->num_sms < kResMaxCtas ? ctx->num_sms : kResMaxCtas;
+    return ctx->res_sms > 0 && ctx->res_sms < ctas ? ctx->res_sms : ctas;
+}
+
+// Whether this device runs an instance as it is meant to: its register split
+// assumes the registers of the launch, and a CTA has to fit on an SM.  Looked
+// up once per context; the blocked kernel serves what does not run here.
+bool res_usable(hp_ctx* ctx, int width, int R)
+{
+    int8_t& known = ctx->res_known[width_class(width)][R / 8];
+    if (known == 0) {
+        const ResKernel k = res_kernel(width, R);
+        cudaFuncAttributes fa;
+        int fit = 0;
+        cudaError_t e =
+            cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k.fn);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k.fn, kResThreads, k.smem);
+        if (e != cudaSuccess) cudaGetLastError();
+        known = e == cudaSuccess && fa.numRegs == kResRegs && fit >= 1 ? 1 : -1;
+    }
+    return known > 0;
+}
 
 // The split with the least time: waves of groups x time per sweep of a strip,
 // measured with all SMs at work and obstacles in every grid (38, 152 and 152
@@ -32,7 +59,7 @@ int res_ctas(const hp_ctx* ctx) { return ctx->num_sms < kResMaxCtas ? ctx->num_s
 // 3.7 and 4.9 us per sweep with 4, 8 and 16 rows (four, two waves and one), one
 // 512^2 grid 1.43, 2.0 and 3.4 us.  64 x 256^2 in one wave of 16 rows took 4.5
 // us a sweep and all grids as long as the slowest; in two of 8 rows 3.6 us.
-bool res_plan(const hp_ctx* ctx, hp_shape s, ResPlan* best)
+bool res_plan(hp_ctx* ctx, hp_shape s, ResPlan* best)
 {
     // wider than 512 cells: columns of 240, eight copied on each side
     const int width = s.nx <= 128 ? 128 : s.nx <= 256 ? 256 : s.nx <= 512 ? 512 : 1024;
@@ -45,12 +72,12 @@ bool res_plan(const hp_ctx* ctx, hp_shape s, ResPlan* best)
     double least = 0.0;
     bool found = false;
     for (int R : {4, 8, 16}) {
-        if (R == 4 && width == 1024) continue;
+        if ((R == 4 && width == 1024) || !res_usable(ctx, width, R)) continue;
         const int rows = res_kernel(width, R).rows, n = (s.ny + rows - 1) / rows * ntx;
         if (n > ctas) continue;
         const int groups = ctas / n < s.batch ? ctas / n : s.batch;
         const int waves = (s.batch + groups - 1) / groups;
-        const double t = waves * us[width == 128 ? 0 : width == 256 ? 1 : width == 512 ? 2 : 3][R / 8];
+        const double t = waves * us[width_class(width)][R / 8];
         if (!found || t < least) {
             least = t;
             *best = {width, R, n, ntx, groups};
@@ -120,12 +147,6 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     if (!res_plan(ctx, s, &p)) return HP_OK;
     if (phi0 == ctx->phi[0]) return HP_ERR_INVALID_ARG;  // see ResArgs::phi
     const ResKernel k = res_kernel(p.width, p.R);
-    cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
-    cudaFuncAttributes fa;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k.fn);
-    // the register split of the kernel assumes what the launch allocates
-    if (e == cudaSuccess && fa.numRegs != kResRegs) e = cudaErrorInvalidKernelImage;
-    if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
     ResArgs a = {};
     a.phi0 = phi0;
     a.phi0_vec = phi0 && ((uintptr_t)phi0 & 15) == 0;
@@ -172,7 +193,12 @@ hp_status launch_resident(hp_ctx* ctx, hp_shape s, double threshold, int cap, bo
     cfg.attrs = at;
     cfg.numAttrs = p.n > 1 ? 1 : 0;  // single CTAs wait for nobody
     void* args[] = {&a};
-    e = cudaLaunchKernelExC(&cfg, k.fn, args);
+    cudaError_t e = cudaLaunchKernelExC(&cfg, k.fn, args);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // fewer SMs for this stream than the device has: the blocked kernel
+        cudaGetLastError();
+        return HP_OK;
+    }
     if (e != cudaSuccess) { set_cuda_error(e); return HP_ERR_CUDA; }
     *launched = true;
     return check_launch();
@@ -192,6 +218,13 @@ int32_t hp_resident_clusters(hp_ctx* ctx, hp_shape s)
     if (!ctx || !hp::shape_ok(s)) return 0;
     const int tiles = ((s.nx + 127) / 128) * ((s.ny + 127) / 128);
     return tiles > 16 ? 0 : hp::resident_capacity(ctx, s);
+}
+
+hp_status hp_ctx_set_resident_sms(hp_ctx* ctx, int32_t sms)
+{
+    if (!ctx || sms < 0) return HP_ERR_INVALID_ARG;
+    ctx->res_sms = sms;
+    return HP_OK;
 }
 
 }  // extern "C"
