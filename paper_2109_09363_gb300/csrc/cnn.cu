@@ -1783,21 +1783,28 @@ __global__ void upsample_adjoint_kernel(const float* __restrict__ gfine, int str
 
 // residual of the scaled problem and per-grid loss sums:
 // {sum_f e, sum_f e^2, N_f, sum r^2, sum_f t, sum_f t^2, sum d^2}
-// with t = target/s, d = div/s, e = phi - t, as kLossCtas partial sums per
-// grid, stats[b][part][kStats], that the readers add in order.  What bounds
+// with t = target/s, d = div/s, e = phi - t, as partial sums of loss_parts CTAs
+// per grid, stats[b][part][kStats], that the readers add in order.  What bounds
 // the loss is the rate of FP64 (about two operations a cycle and SM, 15 per
-// cell here), so the cells of a grid are spread over several SMs, and the
-// gradient's quotients by values of the grid are products with their
-// reciprocals: 64 x 128^2 with one CTA per grid and three FP64 quotients per
-// cell 83 us for the sums and 116 us for the gradient, now 59 and 27 us (cold
-// caches).
+// cell here), so the cells of a grid are spread over several SMs (2,048 cells
+// each or more: 1024 x 16^2 in eight CTAs a grid made the whole gradient 0.2 ms,
+// 2 %, longer), and the gradient's quotients by values of the grid are products
+// with their reciprocals: 64 x 128^2 with one CTA per grid and three FP64
+// quotients per cell 83 us for the sums and 116 us for the gradient, now 59 and
+// 27 us (cold caches).
 constexpr int kStats = 7;
-constexpr int kLossCtas = 8;
+constexpr int kLossCtas = 8;  // at most
 
-__device__ __forceinline__ double loss_stat(const double* __restrict__ stats, int b, int k)
+static int loss_parts(size_t cells)
+{
+    return cells >= 2048 * kLossCtas ? kLossCtas : cells < 2048 ? 1 : (int)(cells / 2048);
+}
+
+__device__ __forceinline__ double loss_stat(const double* __restrict__ stats, int parts, int b,
+                                            int k)
 {
     double t = 0.0;
-    for (int p = 0; p < kLossCtas; ++p) t += stats[((size_t)b * kLossCtas + p) * kStats + k];
+    for (int p = 0; p < parts; ++p) t += stats[((size_t)b * kLossCtas + p) * kStats + k];
     return t;
 }
 
@@ -1812,7 +1819,7 @@ __global__ void loss_stats_kernel(const float* __restrict__ phi, const float* __
     const size_t cells = (size_t)ny * nx, base = (size_t)b * cells;
     const float inv_s = 1.0f / s[b];
     double v[kStats] = {0, 0, 0, 0, 0, 0, 0};
-    for (size_t c = blockIdx.x * blockDim.x + threadIdx.x; c < cells; c += kLossCtas * blockDim.x) {
+    for (size_t c = blockIdx.x * blockDim.x + threadIdx.x; c < cells; c += gridDim.x * blockDim.x) {
         const uint32_t m = mask[base + c];
         const float pc = phi[base + c];
         const float dc = div[base + c] * inv_s;
@@ -1863,13 +1870,13 @@ __global__ void __launch_bounds__(256)
     loss_grad_kernel(const float* __restrict__ phi, const float* __restrict__ target,
                      const float* __restrict__ rbuf, const uint8_t* __restrict__ mask,
                      const uint8_t* __restrict__ flags, const float* __restrict__ s,
-                     const double* __restrict__ stats, float lambda, float* __restrict__ g, int B,
-                     int ny, int nx)
+                     const double* __restrict__ stats, int parts, float lambda,
+                     float* __restrict__ g, int B, int ny, int nx)
 {
     __shared__ double st[kStats], s_mean, s_gain, s_inv;
     __shared__ float s_div;
     const int b = blockIdx.y;
-    if (threadIdx.x < kStats) st[threadIdx.x] = loss_stat(stats, b, threadIdx.x);
+    if (threadIdx.x < kStats) st[threadIdx.x] = loss_stat(stats, parts, b, threadIdx.x);
     __syncthreads();
     if (threadIdx.x == 0) {
         const double nf = st[2], vt = target_var(st), d2 = st[6];
@@ -1912,13 +1919,13 @@ __device__ __forceinline__ double warp_sum_fixed(double v)
 }
 
 // one warp: lane l takes the grids b = l (mod 32) in order
-__global__ void loss_finish_kernel(const double* __restrict__ stats, int B, size_t cells,
-                                   float lambda, double* __restrict__ loss)
+__global__ void loss_finish_kernel(const double* __restrict__ stats, int parts, int B,
+                                   size_t cells, float lambda, double* __restrict__ loss)
 {
     double L = 0.0;
     for (int b = threadIdx.x; b < B; b += 32) {
         double st[kStats];
-        for (int k = 0; k < kStats; ++k) st[k] = loss_stat(stats, b, k);
+        for (int k = 0; k < kStats; ++k) st[k] = loss_stat(stats, parts, b, k);
         const double vt = target_var(st);
         if (st[2] > 0.0 && vt > 0.0) L += (st[1] - st[0] * st[0] / st[2]) / vt;
         if (st[6] > 0.0) L += lambda * st[3] / st[6];
@@ -2805,13 +2812,14 @@ static hp_status trainer_grad(hp_trainer* t, const float* div, const uint8_t* fl
     if ((rc = launch_mask(flags, t->mask, s, st)) != HP_OK) return rc;
     const size_t cells = (size_t)s.ny * s.nx;
     const float* phi = (const float*)t->act[c->nlayers - 1];
-    loss_stats_kernel<<<dim3(kLossCtas, s.batch), 512, 0, st>>>(phi, target, div, t->mask, flags, c->s, t->rbuf,
-                                               t->stats, s.ny, s.nx);
+    const int parts = loss_parts(cells);
+    loss_stats_kernel<<<dim3(parts, s.batch), 512, 0, st>>>(phi, target, div, t->mask, flags, c->s,
+                                                            t->rbuf, t->stats, s.ny, s.nx);
     loss_grad_kernel<<<dim3((unsigned)((cells + kLossCells - 1) / kLossCells), s.batch), 256, 0,
                        st>>>(
-        phi, target, t->rbuf, t->mask, flags, c->s, t->stats, lambda, t->g[0], s.batch, s.ny,
+        phi, target, t->rbuf, t->mask, flags, c->s, t->stats, parts, lambda, t->g[0], s.batch, s.ny,
         s.nx);
-    loss_finish_kernel<<<1, 32, 0, st>>>(t->stats, s.batch, cells, lambda, t->loss);
+    loss_finish_kernel<<<1, 32, 0, st>>>(t->stats, parts, s.batch, cells, lambda, t->loss);
     if ((rc = check_launch()) != HP_OK) return rc;
     return trainer_backward(t, s, st);
 }
