@@ -47,7 +47,8 @@ typedef enum {
     HP_ERR_NONFINITE = 3,   /* the input velocity holds NaN or Inf */
     HP_ERR_OOM = 5,         /* device allocation failed */
     HP_ERR_UNSUPPORTED = 6, /* the requested combination is not built */
-    HP_ERR_TIMEOUT = 7,     /* a bounded device wait gave up (hp_cnn_check, hp_ctx_check) */
+    HP_ERR_TIMEOUT = 7,     /* a bounded device wait gave up: of a tensor-core kernel
+                               (hp_cnn_check) or of the sweeps (hp_ctx_check) */
     HP_ERR_IO = 8,          /* a checkpoint file could not be written, or is missing,
                                truncated, corrupted or of another format version */
     HP_ERR_GUARD = 9,       /* a workspace's guard zone was overwritten (hp_ctx_check,
@@ -88,8 +89,8 @@ typedef struct {
  *                  one on each SM, keep it on chip for all sweeps, falling
  *                  back to 2 for grids that the SMs do not hold (somewhat
  *                  above 2048 x 2048).  All give the same iterates bit for
- *                  bit; the FP64 E_k may differ in the last bits between
- *                  kernels (their partial sums are grouped differently).
+ *                  bit; E_k may differ in its last digits (1e-8 of it)
+ *                  between kernels, which group their sums differently.
  *   open_top       1 = the top boundary (the v faces of row 0) is open to an
  *                  exterior at p = 0: the faces of fluid cells of row 0 are
  *                  open (counted in n, in the divergence and corrected from
@@ -165,8 +166,9 @@ hp_status hp_div_norms(hp_ctx *ctx, const float *u, const float *v, const uint8_
  *   2. phi_0 = phi0 (the CNN guess of the hybrid method; NULL = 0), set to 0
  *      on cells without an open face;
  *   3. k* = first k with E_1(phi_k) <= threshold, else max_iters; the sweeps
- *      are masked Jacobi on the open-face Laplacian, E_1 is summed in FP64
- *      after every sweep in a fixed order;
+ *      are masked Jacobi on the open-face Laplacian, E_1 is summed after
+ *      every sweep in a fixed order (FP32 partial sums of |r|, then FP64
+ *      or, in the grid-resident kernel, pairs of floats);
  *   4. u = u* - grad phi on open faces, 0 on closed faces; p = phi rho0 / dt.
  * A grid whose E_1 is not finite (NaN or Inf in its input) stops at that k
  * with converged = 0; the other grids of the batch are not affected.

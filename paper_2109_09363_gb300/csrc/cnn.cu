@@ -1398,9 +1398,11 @@ __global__ void conv_wgrad_kernel(const GT* __restrict__ gy, const XT* __restric
 // grad[co][ci][t] (oracle order) = sum over chunks of part[k][t][co][ci];
 // bias likewise.  A block of 256 threads serves 32 outputs; thread group j
 // (of 8) sums the chunks k = j (mod 8) as a float pair (the rounding error of
-// every addition, which is exact in FP32, is kept in a second float: 2^-46 of
-// the sum, far below the FP32 result), and the 8 group sums are added in FP64
-// in a fixed order.  With all sums in FP64 the conversions and additions were
+// every addition, which is exact in FP32, is kept in a second float, whose own
+// roundings come to chunks / 8 * 2^-48 of the sum of magnitudes at most; of
+// 600,000 sums of 152 random partials over eight decades none differed from
+// FP64 sums after rounding to FP32), and the 8 group sums are added in FP64 in a
+// fixed order.  With all sums in FP64 the conversions and additions were
 // what bounded it (about two FP64 operations a cycle and SM): the 19 sums of a
 // training gradient of 64 x 128^2 took 0.22 ms more (3.40 -> 3.18 ms in all).
 // Launch with ceil((9 CO CI + CO) / 32) blocks of 256 threads.

@@ -1507,9 +1507,12 @@ hp_status project_impl(hp_ctx* ctx, float* u, float* v, const uint8_t* flags, hp
     const int R = prm->sweep_kernel == 3 ? 2 : 4;
     bool resident = false;
     if (prm->sweep_kernel == 4 || prm->sweep_kernel == 0) {
-        // library choice: the whole grid on chip, one cluster per grid
-        // (measured 1.85x faster than the blocked kernel at 16 x 512^2); the
-        // blocked loop when the grid is larger or the cluster does not fit
+        // library choice: the whole grid on chip, in strips of one SM each.
+        // Against the blocked kernel, us per sweep: 16 x 512^2 3.9 and 9.7, 1 x
+        // 1024^2 2.0 and 3.9, 4 x 1024^2 6.9 and 9.6, 1 x 2048^2 3.6 and 9.0, 64 x
+        // 64 x 600 1.6 and 5.8; whole projections that stop at sweep 0, 3 or 20:
+        // 4 x 1024^2 197, 200, 365 and 194, 209, 380 us, 16 x 640^2 235, 243, 454
+        // and 270, 296, 560 us.  The blocked loop when the SMs do not hold a grid.
         rc = launch_resident(ctx, s, thr, cap, fixed, phi0, e_hist, hist_len, st, &resident);
         if (rc != HP_OK) return rc;
     }

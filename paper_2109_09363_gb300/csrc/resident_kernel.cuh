@@ -4,10 +4,11 @@
 // A grid stays on chip for all of its sweeps.  It is cut into horizontal
 // strips of whole rows, one CTA (one SM) each, up to 512 cells wide; the CTAs
 // of one grid form a group, and one cooperative launch holds as many groups as
-// fit on the device, each working through grids of the batch.  A CTA is 16
-// warps in WX columns of 32 C cells and 16 / WX warp rows; thread (warp, lane)
+// fit on the device, each working through grids of the batch.  A CTA has 8 sweep
+// warps in WX columns of 32 C cells and 8 / WX warp rows; thread (warp, lane)
 // holds R rows x C columns of phi in registers, div and four bits of open-face
-// count per cell sit in shared memory.  Per sweep and warp:
+// count per cell sit in shared memory.  A ninth warp does the E rounds, two more
+// receive the neighbours' rows.  Per sweep and warp:
 //   - the rows next to the warp's block come from shared memory (double
 //     buffered), or, at the edge of the strip, from the neighbouring CTA
 //     through the L2: every 32-bit value travels with the number of its
@@ -15,13 +16,17 @@
 //     no fence or flag is needed;
 //   - warps of the lower half hold their rows bottom up, so that the row at
 //     the strip's edge is register row 0 in every edge warp: it is computed
-//     and sent first, and travels while the other rows are computed; the
-//     receiver issues its load halfway through the sweep;
+//     and sent first, and travels while the other rows are computed;
 //   - groups of rows whose cells all have the open-face count of an
 //     unobstructed row of that column take the update without the closed-face
 //     terms (bit for bit the same result: the left-out product is an exact
 //     zero), the others look 4 - n and 1/n up by the cell's bits.
 // The only barrier of a sweep is the CTA's own.
+//
+// What bounds it: latency, with two sweep warps per scheduler (the registers
+// hold phi, so there is no room for more).  At 16 x 512^2 the schedulers issue in
+// 45 % of their cycles; an instruction waits 1.2 cycles at the CTA barrier, 0.7 for
+// fixed latencies, 0.5 for shared memory and 0.4 for instructions to be fetched.
 //
 // Grids wider than 512 cells are also cut into columns of 240 cells: a CTA then
 // holds 256 columns, the outer 8 on each side copies of its neighbours' cells.
@@ -137,13 +142,13 @@ template <int C, int R, int WX>
 struct ResLayout {
     static constexpr int WY = kResWarps / WX;
     static constexpr int V = C / 4;                                      // 16-byte words per row
-    static constexpr int kDiv = 0;                                       // [16][R][V][32] float4
-    static constexpr int kCode = kDiv + kResWarps * R * V * 512;         // [16][R][32] u32, 4 bits a cell
-    // rows next to a block: [2 parities][16 warps x 2 rows + a zero row][V][32] float4
+    static constexpr int kDiv = 0;                                       // [8][R][V][32] float4
+    static constexpr int kCode = kDiv + kResWarps * R * V * 512;         // [8][R][32] u32, 4 bits a cell
+    // rows next to a block: [2 parities][8 warps x 2 rows + a zero row][V][32] float4
     static constexpr int kRow = kCode + kResWarps * R * 128;
     static constexpr int kRowSlot = V * 512;
     static constexpr int kRowPar = (2 * kResWarps + 1) * kRowSlot;
-    // columns next to a block: [2][16 warps x 2 columns + a zero column][R] float
+    // columns next to a block: [2][8 warps x 2 columns + a zero column][R] float
     static constexpr int kCol = kRow + 2 * kRowPar;
     static constexpr int kColPar = (2 * kResWarps + 1) * R * 4;
     // rows received from the neighbouring CTAs: [2 sides][2 parities][WX][V][32] float4
