@@ -375,8 +375,9 @@ struct ResWarp {
         for (int q = 0; q < C; ++q) dsp[q] = __fsub_rn(phi[0][q], dsp[q]);
         const int s_div = L::kDiv + (wid * R * V * 32 + lane) * 16;
         const int s_code = L::kCode + (wid * R * 32 + lane) * 4;
-        // |r| in four chains, by column; with 16 rows a thread they would be 32
+        // |r| in four chains, by column; with 128 cells a thread they would be 32
         // values long, so every four rows are added up by themselves
+        constexpr bool kSplit = R * C > 64;
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         float sum[2] = {0.0f, 0.0f};
         float s = pending;
@@ -473,7 +474,7 @@ struct ResWarp {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) after(i);
             }
-            if (WITH_E && R == 16) {
+            if (WITH_E && kSplit) {
                 sum[g / 2] = __fadd_rn(sum[g / 2], __fadd_rn(__fadd_rn(acc[0], acc[1]),
                                                              __fadd_rn(acc[2], acc[3])));
                 acc[0] = acc[1] = acc[2] = acc[3] = 0.0f;
@@ -497,8 +498,8 @@ struct ResWarp {
         if (WITH_E) {
             if (lane < kResSums) *wsum = s;
             pending = mute ? 0.0f : __fadd_rn(
-                R == 16 ? sum[0] : __fadd_rn(acc[0], acc[1]),
-                R == 16 ? sum[1] : __fadd_rn(acc[2], acc[3]));
+                kSplit ? sum[0] : __fadd_rn(acc[0], acc[1]),
+                kSplit ? sum[1] : __fadd_rn(acc[2], acc[3]));
         }
     }
     template <bool P>
@@ -969,24 +970,19 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
         sync_grid();
 
         const bool with_e = !a.fixed || a.gs[b].wild == a.epoch;
-        if (!with_e) {
-            for (int j = 0; j < kstar; ++j) {
-                if (WIDE && j > 0 && j % kResGhost == 0) {
-                    w.drain(a);
-                    refresh();
-                }
-                w.template update<false>(phi, pending, nullptr, a);
-                sync_sweepers();
-            }
-            store_cells(a.phi);
-            w.drain(a);
-        } else {
+        constexpr bool kOneLoop = R * C > 64;
+        // sweeps without E: a run of fixed length, or a replay
+        int done = 0;
+        bool alone = !with_e;
+        if (with_e) {
             // Four sweeps at a time; round q needs the sums of sweeps 4q .. 4q+3,
             // the last stored during sweep 4q + 4.  A replay from phi_0 or the
-            // checkpoint at or below k* to phi_{k*} takes the same loop (and
-            // leaves its sums unread): the code of another one, 94 KB with 16
-            // rows, would have to be fetched first, which took as long as five
-            // sweeps (4 x 1024^2, stop at sweep 3: 250 and 200 us).
+            // checkpoint at or below k* to phi_{k*} takes the same loop where a
+            // thread has 128 cells (and leaves its sums unread): the code of the
+            // sweeps without E, 94 KB, would have to be fetched first, which took
+            // as long as five sweeps (4 x 1024^2, stop at sweep 3: 250 and 200
+            // us).  With fewer cells that code is smaller, and the sweeps below
+            // are faster (16 x 512^2: 20.0 and 19.9 ms in all).
             int last = 0, before = 0, cb = 1;  // latest checkpoints, buffer of the latest
             bool replay = false;
             for (int k = 0;; k += 4) {
@@ -1001,22 +997,25 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     const int base = kstar >= last ? last : before;
                     load_cells(base == 0 ? a.phi0 : a.ck[base == last ? cb : cb ^ 1], base == 0,
                                vec && (base != 0 || a.phi0_vec));
-                    k = base;
-                    replay = loaded = true;
                     sync_sweepers();
                     if (!WIDE || base == 0) {
                         w.publish(phi);
                         sync_sweepers();
                     }
+                    if (!kOneLoop) {
+                        if (WIDE && base > 0) refresh();
+                        done = base;
+                        alone = true;
+                        break;
+                    }
+                    k = base;
+                    replay = loaded = true;
                 }
-                // of the four: sweeps to do, and phi to be kept before one of them
                 const int todo = (replay ? kstar : a.cap + 1) - k;
-                int keep_at = replay ? todo : todo - 1;
-                float* keep = a.phi;
-                if (keep_at > 3 && !replay && k == last + ckpt_step(last)) {
+                const int keep_at = replay ? todo : todo - 1;
+                if (!replay && k == last + ckpt_step(last) && k <= a.cap) {
                     cb ^= 1;
-                    keep = a.ck[cb];
-                    keep_at = 0;
+                    store_cells(a.ck[cb]);
                     before = last;
                     last = k;
                 }
@@ -1052,7 +1051,7 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     }
                     float* wsum = s_wsum + (((k + i - 1 + 4 * (int)first) & (kWsumRing - 1)) * kResWarps +
                                             w.wid) * kResSums + w.lane;
-                    if (i == keep_at) store_cells(keep);
+                    if (i == keep_at) store_cells(a.phi);
                     if (i < todo) {
                         w.template update<true>(phi, pending, wsum, a);
                     } else if (replay) {
@@ -1072,6 +1071,18 @@ __global__ void __launch_bounds__(kResThreads, 1) sweep_resident_kernel(const Re
                     break;
                 }
             }
+        }
+        if (alone) {
+            for (int j = done; j < kstar; ++j) {
+                if (WIDE && j > done && j % kResGhost == 0) {
+                    w.drain(a);
+                    refresh();
+                }
+                w.template update<false>(phi, pending, nullptr, a);
+                sync_sweepers();
+            }
+            store_cells(a.phi);
+            w.drain(a);
         }
         if (threadIdx.x == 0 && rank == 0) {
             GridState* gs = a.gs + b;
