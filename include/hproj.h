@@ -136,7 +136,7 @@ void hp_ctx_destroy(hp_ctx *ctx);
 hp_status hp_ctx_check(hp_ctx *ctx);
 
 /* Polls after which a wait of the grid-resident sweeps gives up, for calls
- * launched from now on; 0 = the compiled limits (about a second).  Its strips
+ * launched from now on; 0 = the compiled limits (about ten seconds).  Its strips
  * wait for one another's rows, and a wait can run out when the device runs
  * some of them much later than the others. */
 hp_status hp_ctx_set_wait_limit(hp_ctx *ctx, uint32_t polls);

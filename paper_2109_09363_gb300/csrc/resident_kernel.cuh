@@ -80,11 +80,12 @@ constexpr int kResRing = 4;        // > kResLag: rounds between the sweeps and t
 constexpr int kWsumRing = 4 * kResRing;  // warp sums, by sweep
 constexpr int kResSums = 4;        // of one warp: each over eight lanes
 // A wait gives up after so many polls: of a word in the L2 (a round trip, half
-// a microsecond, so about a second) or of a barrier (suspended for a microsecond
-// at most); of a word in shared memory, which waits for a warp that waits for
-// the others.  The CTA then marks the launch, waits no longer than one poll
+// a microsecond, so about ten seconds) or of a barrier (suspended for a
+// microsecond at most); of a word in shared memory, which waits for a warp that
+// waits for the others.  Long enough for a CTA that starts late because kernels
+// of other streams hold its SM.  The CTA then marks the launch, waits no longer than one poll
 // each for the rest of its grid (whose result is void) and takes no other grid.
-constexpr int kResPolls = 1 << 21, kResLooks = 1 << 27;
+constexpr int kResPolls = 1 << 24, kResLooks = 1 << 30;
 // the sums of pairs are scaled (exactly) so that no sum of finite warp sums overflows
 constexpr float kSumScale = 1.0f / 8192.0f;
 static_assert(kResMaxCtas * kResWarps * kResSums <= 8192, "FP32 sums of one grid");

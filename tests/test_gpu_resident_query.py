@@ -14,7 +14,11 @@ torch = pytest.importorskip("torch")
 hp = pytest.importorskip("paper_2109_09363_gb300")
 
 
-@pytest.mark.parametrize("shape,grids", [((1, 512, 512), 4), ((16, 512, 512), 9), ((2, 100, 600), 25),
+# (the counts tell 4, 8 or 16 rows a thread apart: an instance that the device
+# does not run as it is meant to would show as another count)
+@pytest.mark.parametrize("shape,grids", [((1, 128, 128), 38), ((70, 128, 128), 76),
+                                         ((1, 256, 256), 19), ((38, 256, 256), 38),
+                                         ((1, 512, 512), 4), ((16, 512, 512), 9), ((2, 100, 600), 25),
                                          ((1, 2048, 2048), 1), ((1, 2600, 2600), 0),
                                          ((1, 20000, 64), 0)])
 def test_query_is_the_launch(dev, shape, grids):  # noqa: F811
